@@ -604,7 +604,12 @@ static paco_status_t build_device(paco_plan *pl, BatchedState *bs)
         smem = std::max(smem, stage_smem_bytes(c.lg2, 13 - c.lg2, 2));
     }
     bs->smem = smem;
-    PACO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the attribute belongs to the kernel, not to the plan: set to what any
+    // configuration needs, so that a second plan does not lower the first one's
+    int most = smem;
+    for (int lgL = batched::STAGE_MIN_LG; lgL <= batched::STAGE_MAX_LG; ++lgL)
+        most = std::max(most, std::max(stage_smem_bytes(lgL, 13 - lgL, 1), stage_smem_bytes(lgL, 13 - lgL, 2)));
+    PACO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     int occ = 0;
     PACO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, batched::NT, smem));
     if (occ < 1) return fail(PACO_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
