@@ -139,6 +139,10 @@ typedef struct {
                                     items_per_pair, h and mu then refer to the
                                     pipeline's second factor N2 N3) */
     int64_t N3;                  /* dims = 3: the third axis; 1 otherwise */
+    int passes;                  /* launches of paco_execute when it runs as passes over
+                                    factors of N chosen for the machine (plain complex64
+                                    plans with no stage option set); 0: the two stages
+                                    described above */
 } paco_plan_info_t;
 
 /*

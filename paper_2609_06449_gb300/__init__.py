@@ -94,6 +94,7 @@ class PlanInfo(ctypes.Structure):
         ("stage_split", ctypes.c_int * 2),
         ("dims", ctypes.c_int),
         ("N3", ctypes.c_int64),
+        ("passes", ctypes.c_int),
     ]
 
 

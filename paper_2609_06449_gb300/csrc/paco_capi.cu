@@ -353,6 +353,7 @@ static paco_status_t plan_build(paco_plan **out, const paco_plan_opts_t *o, int 
     pl->lgLa3 = lgLa3;
     pl->N3 = (o->dims == 3) ? o->N2 >> lgLa3 : 1;
     pl->req_ctas = o->ctas_per_sm;
+    pl->req_tile = o->tile_w != 0 || o->cluster != 0;
     pl->form = (o->dtype == PACO_C64_TC_BF16X3) ? TC_BF16X3 : (o->dtype == PACO_C64_TC_FP16) ? TC_FP16 : TC_NONE;
     if (pl->form) {
         paco_status_t ts = tc_table_create(pl->form, &pl->tc);
@@ -394,6 +395,10 @@ static paco_status_t plan_build(paco_plan **out, const paco_plan_opts_t *o, int 
             return st;
         }
         pl->fused = 1;
+    }
+    if ((st = route_setup(pl)) != PACO_OK) {
+        paco_plan_destroy(pl);
+        return st;
     }
     size_t scratch_elems = 0, words = 0;
     for (int k = 0; k < 2; ++k) {
@@ -451,6 +456,7 @@ extern "C" void paco_plan_destroy(paco_plan_t *pl)
 {
     if (!pl) return;
     batched_destroy(pl->bs);
+    route_destroy(pl->route);
     restore_destroy(pl);
     cudaFree(pl->tc);
     cudaFree(pl->twL1);
@@ -492,6 +498,7 @@ extern "C" paco_status_t paco_plan_info(const paco_plan_t *pl, paco_plan_info_t 
     info->stage_split[0] = pl->st[0].split;
     info->stage_split[1] = pl->st[1].split;
     info->dims = pl->dims;
+    info->passes = route_passes(pl);
     for (int s = 0; s < 2; ++s) {
         info->stage_tile_w[s] = 1 << pl->st[s].lgW;
         info->stage_cluster[s] = 1 << pl->st[s].lgK;
@@ -690,6 +697,13 @@ static void set_device(const paco_plan *pl)
     if (d != pl->device) cudaSetDevice(pl->device);
 }
 
+// paco_debug_set_waits is there to run the stage pipeline's waits out: with it
+// set, a plan with panel stages runs them.
+static bool use_route(const paco_plan *pl)
+{
+    return route_passes(pl) && !((pl->st[0].panel || pl->st[1].panel) && (pl->dbg_wait_bias || pl->dbg_spin_limit));
+}
+
 extern "C" paco_status_t paco_execute(paco_plan_t *pl, const void *in, void *out, int dir,
                                       paco_stream_t stream)
 {
@@ -699,6 +713,7 @@ extern "C" paco_status_t paco_execute(paco_plan_t *pl, const void *in, void *out
     cudaStream_t s = (cudaStream_t)stream;
     if (pl->bs) return batched_execute(pl, in, out, dir, s);
     if (pl->fused) return launch_cluster(pl, in, out, dir, nullptr, s);
+    if (use_route(pl)) return route_run(pl, in, out, dir, nullptr, s);
     if ((st = launch_stage(pl, pl->st[0], 1, in, out, dir, s)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[1], 2, out, out, dir, s);
 }
@@ -848,7 +863,10 @@ extern "C" paco_status_t paco_execute_weighted_power(paco_plan_t *pl, const void
     t.st_w = w;
     t.st_loss = loss;
     t.st_weighted = out_weighted ? 1 : 0;
-    if ((st = launch_stage(pl, pl->st[0], 1, in, out, dir, s)) != PACO_OK) return st;
+    st = route_has_power(pl, 0) ? route_power(pl, 0, in, out, dir, t, s)
+                                : launch_stage(pl, pl->st[0], 1, in, out, dir, s);
+    if (st != PACO_OK) return st;
+    if (route_has_power(pl, 1)) return route_power(pl, 1, out, out, dir, t, s);
     return launch_stage(pl, pl->st[1], 2, out, out, dir, s, &t);
 }
 
@@ -870,6 +888,7 @@ extern "C" paco_status_t paco_execute_weighted_input(paco_plan_t *pl, const void
     t.ld_scale = scale;
     t.ld_mult = mult;
     t.ld_on = 1;
+    if (use_route(pl) && !w) return route_run(pl, in, out, dir, &t, s);
     if ((st = launch_stage(pl, pl->st[0], 1, in, out, dir, s, &t)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[1], 2, out, out, dir, s);
 }

@@ -32,6 +32,8 @@ struct StageCfg {
 };
 
 struct BatchedState;  // paco_batched.cu
+struct Route;         // paco_route.cu
+struct StageTerms;    // paco_stage_args.cuh
 
 } // namespace paco
 
@@ -53,6 +55,8 @@ struct paco_plan {
     int form = 0;                  // tensor-core precision form (paco_tc.cuh), 0 = plain
     int req_ctas = 0;              // requested CTAs per SM of the stage kernels (0 = default)
     int req_split = 0;             // paco_plan_opts_t.split
+    int req_tile = 0;              // 1: a tile width or cluster size was asked for
+    paco::Route *route = nullptr;  // the passes of paco_execute (paco_route.cu), or nullptr: the stage kernels
     int dims = 1;                  // 2: the 2-D DFT (the top-level twiddle tables hold ones)
     int64_t N3 = 1;                // dims = 3: the third axis; N2 (the pipeline's factor) is N2' N3
     int lgLa3 = 0;                 // dims = 3: log2 of the middle axis N2' (Phase III's first split pass)
@@ -94,6 +98,18 @@ bool cluster_eligible(const paco_plan *pl);
 paco_status_t cluster_setup(paco_plan *pl);
 paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int dir, unsigned *pair_count,
                              cudaStream_t stream);
+
+// paco_route.cu
+paco_status_t route_setup(paco_plan *pl);
+void route_destroy(Route *r);
+int route_passes(const paco_plan *pl);
+// terms: the scalar factor of the input, or nullptr
+paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir, const StageTerms *terms,
+                        cudaStream_t stream);
+// one stage (0, 1) of the weighted power: Phase I, and Phase III with the sum
+bool route_has_power(const paco_plan *pl, int stage);
+paco_status_t route_power(const paco_plan *pl, int stage, const void *in, void *out, int dir, const StageTerms &terms,
+                          cudaStream_t stream);
 
 // paco_restore.cu
 paco_status_t restore_setup(paco_plan *pl);
