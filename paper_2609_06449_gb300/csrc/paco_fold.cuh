@@ -1,0 +1,402 @@
+// paco_fold.cuh -- a local-FFT pass with the inter-pass twiddles inside its
+// butterflies.
+//
+// A transform of N points taken digit by digit, most significant input digit
+// first, needs at every radix-2 level one factor per butterfly,
+// w_{2M}^{-kappa} with M the number of frequencies found so far and kappa in
+// [M] this one's index.  Written as
+//     p = E + t O   (four fused multiply-adds),   E - t O = 2 E - p   (two)
+// a level costs three operations a point, twiddle included, against the 2.6 of
+// a radix-16 or -32 DFT plus the four of a separate complex product; nothing
+// is multiplied on its way out of a pass, so Phase I stores plain DFTs and the
+// top-level twiddle w_N^{-k1 c} (Sect. 3.3) is taken by Phase III's
+// butterflies.  In complex128, which the FP64 pipe bounds, the count is the
+// time (2^27: 109 operations a point and 27.5 ms with separate products in the
+// stage kernels).  In complex64 it is the issue rate: a pass of 1024 points
+// over 2^28 went from 1.38 ms (139 instructions a point) to 0.76-0.93 ms.
+//
+// A pass transforms L = A B rows (j = j_hi B + j_lo, k = k_lo + A k_hi) of a
+// tile of W columns: A-point DFTs over j_hi in registers, one exchange through
+// shared memory, B-point DFTs over j_lo.  FIRST: kappa = 0, column c of the
+// view is stored as row pi(c) of the result (the one redistribution).  Else
+// the pass runs in place on row blocks, its columns are the frequencies found
+// so far (kappa = column, K of them), and rows are read through pi.
+//
+// Twiddles (TW).  0: kappa = 0 (the first pass; every pass of the 2-D and 3-D
+// forms): plain DFTs, w_L^{-k_lo j_lo} between them.  1: all of the pass's
+// factors come, rounded once from FP64, out of one table of about K L / 2
+// entries, a level's factors being a run in kappa.  2, where that table would
+// not stay in L2 (K L > 2^20): F1's factors and w_{K L}^{-kappa 2^i} are set up
+// per tile in shared memory, rounded once, and a factor of F2 is one more
+// product of such a value with w_L's.
+//
+// The folded butterflies multiply at every level, so the rounding of their
+// factors shows: with all factors as products of rounded values the relative
+// error of 2^24 points is 2.2e-7, with the tables above 1.9e-7 (the stage
+// kernels: 2.0e-7).  2 E - p carries p's rounding on; in FP64, whose error is
+// held to the stage kernels' too, TW 1 therefore multiplies F1's rows first
+// and takes the plain DFT (ROWS).
+#pragma once
+
+#include "paco_common.cuh"
+
+namespace paco {
+
+template <typename R>
+struct FoldArgs {
+    const cx<R> *in;
+    cx<R> *out;
+    long long bstride;      // elements between two transforms
+    unsigned rowA[32];      // element offset of input row (j_hi B) under the row map
+    unsigned rowK[32];      // element offset of output row A k_hi (not FIRST)
+    unsigned ld_in, ld_out; // elements between two rows
+    int rev_bits, rev_t;    // row map of j_lo: pi over rev_bits bits (0: natural rows)
+    int crev_bits, crev_t;  // FIRST: row pi(c) of column c
+    int lg_tiles;           // log2 of the column tiles of one row block
+    int lg_all;             // log2 of the tiles of one transform
+    unsigned blk_stride;    // elements between two row blocks
+    const cx<R> *tau;       // the factors: F1's then F2's (TW 0: F2's, TW 2: F2's for kappa = 0)
+    const cx<double> *lo;   // TW 2: w_N^{-r}, r < 2^lo_bits
+    const cx<double> *hi;   //       w_N^{-(r << lo_bits)}
+    int lo_bits;
+    int lg_n, lg_k;         // log2 N, log2 K
+    int conj;               // 1: the conjugate transform
+    R mult;                 // FIRST: the input is scaled by mult * (*scale or 1)
+    const double *scale;
+};
+
+template <typename R> struct vec2;
+template <> struct vec2<float> { using type = float2; };
+template <> struct vec2<double> { using type = double2; };
+
+__device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// (e, o) -> (e + t o, e - t o), the second as 2 e - (e + t o) or (DIRECT) on its
+// own: two more operations, and p's rounding is not carried on.
+template <bool DIRECT, typename R>
+__device__ __forceinline__ void bfly(cx<R> &e, cx<R> &o, cx<R> t)
+{
+    const R px = fma_r(-t.y, o.y, fma_r(t.x, o.x, e.x)), py = fma_r(t.y, o.x, fma_r(t.x, o.y, e.y));
+    if constexpr (DIRECT)
+        o = make_cx<R>(fma_r(t.y, o.y, fma_r(-t.x, o.x, e.x)), fma_r(-t.y, o.x, fma_r(-t.x, o.y, e.y)));
+    else
+        o = make_cx<R>(fma_r(R(2), e.x, -px), fma_r(R(2), e.y, -py));
+    e = make_cx<R>(px, py);
+}
+
+// a * w_32^{-E}
+template <int E, typename R>
+__device__ __forceinline__ cx<R> mul_w32(cx<R> a)
+{
+    constexpr R c1 = R(0.98078528040323044912618223613424), s1 = R(0.19509032201612826784828486847702);
+    constexpr R c2 = R(PACO_C8), s2 = R(PACO_S8);
+    constexpr R c3 = R(0.83146961230254523707878837761791), s3 = R(0.55557023301960222474283081394853);
+    constexpr int q = E & 31;
+    if constexpr (q == 0) return a;
+    else if constexpr (q == 1) return mul_const(a, c1, -s1);
+    else if constexpr (q == 2) return mul_const(a, c2, -s2);
+    else if constexpr (q == 3) return mul_const(a, c3, -s3);
+    else if constexpr (q == 4) return mul_w8_1(a);
+    else if constexpr (q == 5) return mul_const(a, s3, -c3);
+    else if constexpr (q == 6) return mul_const(a, s2, -c2);
+    else if constexpr (q == 7) return mul_const(a, s1, -c1);
+    else return mul_mi(mul_w32<q - 8>(a));
+}
+
+template <int S, int R_, typename R>
+__device__ __forceinline__ void tw32_row(cx<R> *v)
+{
+    if constexpr (R_ < 8) {
+        v[S * 8 + R_] = mul_w32<S * R_>(v[S * 8 + R_]);
+        tw32_row<S, R_ + 1>(v);
+    }
+}
+
+// 32-point DFT: radix 4 over r, r + 8, r + 16, r + 24, twiddle w_32^{-s r},
+// radix 8 over r; k = s + 4 m.
+template <typename R>
+__device__ __forceinline__ void dft32(cx<R> *v)
+{
+#pragma unroll
+    for (int r = 0; r < 8; ++r) dft4_s(v[r], v[r + 8], v[r + 16], v[r + 24]);
+    tw32_row<1, 1>(v);
+    tw32_row<2, 1>(v);
+    tw32_row<3, 1>(v);
+    cx<R> y[32];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        dft8(v + 8 * s);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) y[s + 4 * m] = v[8 * s + m];
+    }
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = y[k];
+}
+
+// the plain DFT of a pass without twiddles
+template <int RADIX, typename R>
+__device__ __forceinline__ void plain_dft(cx<R> *v)
+{
+    if constexpr (RADIX == 32) dft32(v);
+    else dft<RADIX>(v);
+}
+
+// One level: size n of an RADIX-point DFT held in bit-reversed order in u.
+// tau(q) with q = tau_index(n, s) is T^(RADIX / n) w_n^{-s}, s < n / 4 (s = 0 for n = 2, 4).
+__host__ __device__ constexpr int tau_index(int n, int s) { return n == 2 ? 0 : n / 4 + s; }
+
+template <bool DIRECT, typename R, int RADIX, int N_, class Tau>
+__device__ __forceinline__ void fold_level(cx<R> *u, const Tau &tau)
+{
+    constexpr int Q = N_ >= 4 ? N_ / 4 : 1;
+#pragma unroll
+    for (int s = 0; s < Q; ++s) {
+        const cx<R> t = tau(tau_index(N_, s));
+#pragma unroll
+        for (int b = 0; b < RADIX; b += N_) {
+            bfly<DIRECT>(u[b + s], u[b + s + N_ / 2], t);
+            if constexpr (N_ >= 4) bfly<DIRECT>(u[b + s + Q], u[b + s + Q + N_ / 2], make_cx<R>(t.y, -t.x));
+        }
+    }
+    if constexpr (N_ < RADIX) fold_level<DIRECT, R, RADIX, N_ * 2>(u, tau);
+}
+
+template <int RADIX>
+__host__ __device__ constexpr int bitrev_c(int i)
+{
+    int r = 0;
+    for (int b = 1; b < RADIX; b <<= 1) r = (r << 1) | ((i & b) ? 1 : 0);
+    return r;
+}
+
+// v[k] = sum_r v[r] T^r w_RADIX^{-rk}
+template <bool DIRECT, typename R, int RADIX, class Tau>
+__device__ __forceinline__ void fold_dft(cx<R> *v, const Tau &tau)
+{
+    cx<R> u[RADIX];
+#pragma unroll
+    for (int i = 0; i < RADIX; ++i) u[i] = v[bitrev_c<RADIX>(i)];
+    fold_level<DIRECT, R, RADIX, 2>(u, tau);
+#pragma unroll
+    for (int i = 0; i < RADIX; ++i) v[i] = u[i];
+}
+
+template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_>
+struct FoldCfg {
+    using R = R_;
+    static constexpr int LGA = LGA_, LGB = LGB_, LGW = LGW_;
+    static constexpr bool FIRST = FIRST_;
+    static constexpr int TW = FIRST_ ? 0 : TW_;
+    static constexpr int A = 1 << LGA, B = 1 << LGB, W = 1 << LGW, L = A * B;
+    static constexpr int EPT = A > B ? (A > 16 ? A : 16) : (B > 16 ? B : 16);
+    static constexpr int NT = L * W / EPT;
+    static constexpr int U1 = EPT / A, U2 = EPT / B;
+    // exchange layouts as in paco_pass.cuh; PH points make one shared-memory phase
+    static constexpr int PH = sizeof(R) == 4 ? 16 : 8;
+    static constexpr int SJ = FIRST ? A + 1 : W;
+    static constexpr int SC0 = B * SJ;
+    static constexpr int SC = FIRST ? SC0 + (((W < PH ? PH / W : 1) - SC0 % PH + PH) % PH) : 1;
+    static constexpr int SK = FIRST ? 1 : B * W + (W < PH ? (W - (B * W) % PH + PH) % PH : 0);
+    static constexpr int EX = FIRST ? W * SC : A * SK;
+    static constexpr bool FP64 = sizeof(R) == 8;
+    static constexpr bool ROWS = TW && FP64;                      // F1's factors by row (T^r), not by level
+    static constexpr int NA = ROWS ? A : A / 2;                   // factors of F1, a column
+    static constexpr int NTW = TW == 2 ? (NA + LGB) * W : 0;
+    static constexpr int SMEM = (EX + NTW) * 2 * (int)sizeof(R);
+    static constexpr int REGS = EPT * 2 * (int)sizeof(R) / 4 + (sizeof(R) == 4 ? (EPT == 32 ? 64 : 32) : 64);
+    static constexpr int REGS_CTAS = 65536 / (REGS * NT);
+    static constexpr int SMEM_CTAS = (227 * 1024) / (SMEM + 1024);
+    static constexpr int MINB = REGS_CTAS < 1 ? 1 : (REGS_CTAS < SMEM_CTAS ? REGS_CTAS : SMEM_CTAS);
+};
+
+template <class CFG>
+__global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __grid_constant__ FoldArgs<typename CFG::R> a)
+{
+    using R = typename CFG::R;
+    using C = cx<R>;
+    using V = typename vec2<R>::type;
+    constexpr int A = CFG::A, B = CFG::B, W = CFG::W, NT = CFG::NT, U1 = CFG::U1, U2 = CFG::U2;
+    constexpr bool FIRST = CFG::FIRST;
+    constexpr int TW = CFG::TW;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *sm = reinterpret_cast<C *>(smem_raw);
+    [[maybe_unused]] C *tabA = sm + CFG::EX;       // TW 2: [tau index][col]
+    [[maybe_unused]] C *tabB = tabA + CFG::NA * W; //       [i][col]: w_{K L}^{-kappa 2^i}
+    const int tid = threadIdx.x;
+    const int tile = (int)(blockIdx.x & ((1u << a.lg_all) - 1u));
+    const long long boff = (long long)(blockIdx.x >> a.lg_all) * a.bstride;
+    const int blk = FIRST ? 0 : tile >> a.lg_tiles;
+    const unsigned c0 = (unsigned)(FIRST ? tile : tile & ((1 << a.lg_tiles) - 1)) << CFG::LGW;
+    const long long base = boff + (long long)blk * (FIRST ? 0u : a.blk_stride) + c0;
+
+    // TW 2: the columns' factors (exponents of w_N, all below N), used while the
+    // tile is on its way.  With 32 points a thread their table reads go out
+    // before the tile's (1024 points 0.93 -> 0.87 ms per 2^28, 512: 0.78 -> 0.75);
+    // with 16 the address work would hold up too many small tiles (256: 0.65, 0.68).
+    constexpr int NI = (CFG::NTW + NT - 1) / NT;
+    [[maybe_unused]] double2 twl[NI ? NI : 1], twh[NI ? NI : 1];
+    [[maybe_unused]] auto load_twiddles = [&] {
+#pragma unroll
+        for (int k = 0; k < NI; ++k) {
+            const int e = tid + NT * k, i = e >> CFG::LGW;
+            const unsigned kap = c0 + (e & (W - 1));
+            unsigned x;
+            if (i < CFG::NA) {                               // i = tau_index(n, s)
+                const int lgq = i ? 31 - __clz(i) : 0, lgn = i ? lgq + 2 : 1, s = i ? i - (1 << lgq) : 0;
+                x = ((kap + ((unsigned)s << a.lg_k)) << (CFG::LGA - lgn)) << (a.lg_n - a.lg_k - CFG::LGA);
+            } else {
+                x = (kap << (i - CFG::NA)) << (a.lg_n - a.lg_k - CFG::LGA - CFG::LGB);
+            }
+            if (CFG::NTW % NT == 0 || e < CFG::NTW) {
+                if constexpr (sizeof(R) == 8) {              // rounded once, in the table
+                    twl[k] = __ldg(reinterpret_cast<const double2 *>(a.tau) + CFG::L / 2 + ((unsigned)i << a.lg_k) + kap);
+                    continue;
+                }
+                twl[k] = __ldg(reinterpret_cast<const double2 *>(a.lo + (x & ((1u << a.lo_bits) - 1u))));
+                twh[k] = __ldg(reinterpret_cast<const double2 *>(a.hi + (x >> a.lo_bits)));
+            }
+        }
+    };
+    if constexpr (TW == 2 && CFG::EPT == 32) load_twiddles();
+
+    // ---- F1
+    C v[CFG::EPT];
+#pragma unroll
+    for (int u = 0; u < U1; ++u) {
+        const int s = tid + NT * u, col = s & (W - 1), jlo = s >> CFG::LGW;
+        const unsigned jrow = a.rev_bits ? digit_reverse((unsigned)jlo, a.rev_bits, a.rev_t) : (unsigned)jlo;
+        const V *p = reinterpret_cast<const V *>(a.in + base + col + (long long)jrow * a.ld_in);
+        if (a.conj) {
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                const V t = __ldcg(p + a.rowA[r]);
+                v[u * A + r] = make_cx<R>(t.y, t.x);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                const V t = __ldcg(p + a.rowA[r]);
+                v[u * A + r] = make_cx<R>(t.x, t.y);
+            }
+        }
+    }
+    if constexpr (TW == 2) {
+        if constexpr (CFG::EPT != 32) load_twiddles();
+#pragma unroll
+        for (int k = 0; k < NI; ++k)
+            if (CFG::NTW % NT == 0 || tid + NT * k < CFG::NTW) {
+                cx<double> t = make_cx<double>(twl[k].x, twl[k].y);
+                if constexpr (sizeof(R) == 4) t = cmul(t, make_cx<double>(twh[k].x, twh[k].y));
+                tabA[tid + NT * k] = make_cx<R>((R)t.x, (R)t.y);
+            }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < U1; ++u) {
+        const int s = tid + NT * u, col = s & (W - 1), jlo = s >> CFG::LGW;
+        const V *t1 = reinterpret_cast<const V *>(a.tau);
+        C *ex = sm + (FIRST ? col * CFG::SC + jlo * CFG::SJ : jlo * W + col);
+        if constexpr (TW == 0) {
+            plain_dft<A>(v + u * A);
+            if constexpr (CFG::FP64) {
+#pragma unroll
+                for (int k = 1; k < A; ++k) {
+                    const V t = __ldg(t1 + k * jlo);         // w_L^{-k_lo j_lo}
+                    v[u * A + k] = cmul(v[u * A + k], make_cx<R>(t.x, t.y));
+                }
+            }
+        } else {
+            t1 += c0 + col;
+            auto f1 = [&](int q) {
+                if constexpr (TW == 2) return tabA[q * W + col];
+                const V t = __ldg(t1 + ((unsigned)q << a.lg_k));
+                return make_cx<R>(t.x, t.y);
+            };
+            if constexpr (CFG::ROWS) {
+#pragma unroll
+                for (int r = 1; r < A; ++r) v[u * A + r] = cmul(v[u * A + r], f1(r));
+                plain_dft<A>(v + u * A);
+            } else {
+                fold_dft<false, R, A>(v + u * A, f1);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < A; ++k) ex[FIRST ? k : k * CFG::SK] = v[u * A + k];
+    }
+    __syncthreads();
+    // ---- F2
+#pragma unroll
+    for (int u = 0; u < U2; ++u) {
+        const int s = tid + NT * u;
+        int col, klo;
+        if constexpr (FIRST) { klo = s & (A - 1); col = s >> CFG::LGA; }
+        else { col = s & (W - 1); klo = s >> CFG::LGW; }
+        const C *ex = sm + (FIRST ? col * CFG::SC + klo : klo * CFG::SK + col);
+#pragma unroll
+        for (int r = 0; r < B; ++r) v[u * B + r] = ex[r * CFG::SJ];
+        if constexpr (TW == 0 && CFG::FP64) {
+            plain_dft<B>(v + u * B);
+        } else {
+            // factor q of (k_lo, column): entry q A + k_lo after F1's
+            const V *t2 = reinterpret_cast<const V *>(a.tau);
+            if constexpr (TW == 1) t2 += c0 + col + ((unsigned)(CFG::NA + klo) << a.lg_k);
+            else t2 += klo;
+            fold_dft<TW != 1 && !CFG::FP64, R, B>(v + u * B, [&](int q) {
+                const V t = __ldg(t2 + (TW == 1 ? (unsigned)(q * A) << a.lg_k : (unsigned)(q * A)));
+                const C w = make_cx<R>(t.x, t.y);
+                if constexpr (TW != 2) return w;
+                int lg = 0;                                  // B / n = 2^lg
+                while ((q == 0 ? 2 : 4 << (31 - __clz(q))) << lg < B) ++lg;
+                return cmul(w, tabB[lg * W + col]);
+            });
+        }
+        V *q;
+        if constexpr (FIRST) {
+            const unsigned c = c0 + col;
+            const unsigned row = a.crev_bits ? digit_reverse(c, a.crev_bits, a.crev_t) : c;
+            q = reinterpret_cast<V *>(a.out + boff + (long long)row * a.ld_out + klo);
+            const R f = a.scale ? a.mult * (R)__ldg(a.scale) : a.mult;
+            if (f != R(1)) {
+#pragma unroll
+                for (int k = 0; k < B; ++k) v[u * B + k] = make_cx<R>(v[u * B + k].x * f, v[u * B + k].y * f);
+            }
+        } else {
+            q = reinterpret_cast<V *>(a.out + base + col + (long long)klo * a.ld_out);
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const C y = v[u * B + k];
+            V o;
+            o.x = a.conj ? y.y : y.x;
+            o.y = a.conj ? y.x : y.y;
+            q[FIRST ? (unsigned)(A * k) : a.rowK[k]] = o;
+        }
+    }
+}
+
+// What the host needs to launch one of the kernels above.
+struct FoldKernel {
+    const void *fn = nullptr;
+    int lgA = 0, lgB = 0, lgW = 0, threads = 0, smem = 0;
+};
+
+template <class CFG>
+FoldKernel fold_kernel_of()
+{
+    FoldKernel k;
+    k.fn = reinterpret_cast<const void *>(&paco_fold_kernel<CFG>);
+    k.lgA = CFG::LGA;
+    k.lgB = CFG::LGB;
+    k.lgW = CFG::LGW;
+    k.threads = CFG::NT;
+    k.smem = CFG::SMEM;
+    return k;
+}
+
+// The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
+// (the row stride); fn == nullptr where none is built.
+FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC);
+FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC);
+
+} // namespace paco

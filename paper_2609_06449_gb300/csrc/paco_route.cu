@@ -1,35 +1,40 @@
-// paco_route.cu -- how paco_execute runs a complex64 transform: two or three
-// passes of paco_pass.cuh.
+// paco_route.cu -- how paco_execute runs a plan: two to four passes of
+// paco_fold.cuh.
 //
 // The route is the paper's composition Phase I -> redistribution -> Phase III
-// with the two factors chosen for the machine: a pass of up to 2^10 points
-// keeps its tile in one CTA and runs near the copy rate, so a transform of up
-// to 2^20 points takes two of them and a longer one three (Phase III's length
-// L2 L3 split once more, both halves in place in the output).  The result does
-// not depend on the factors (Theorem 3); the plan's own N1, N2 and W stay what
-// paco_execute_stage1 / _stage2 / _phase1 use.
+// with the factors chosen for the machine: a pass keeps its tile in one CTA,
+// so a transform takes ceil(log2 N / 10) of them (complex64; 9 for complex128),
+// the first with the redistribution in its stores, the others in place in the
+// output (Phase III's length split further, Sect. 4.1).  The result does not
+// depend on the factors (Theorem 3); the plan's own N1, N2 and W stay what
+// paco_execute_stage1 / _stage2 / _phase1 use.  The weighted power runs the
+// plan's own two stages (paco_power.cuh).
 #include <cuda_runtime.h>
 
 #include <cstring>
 #include <new>
 
 #include "paco_common.cuh"
-#include "paco_pass.cuh"
+#include "paco_fold.cuh"
+#include "paco_power.cuh"
 #include "paco_plan.h"
 #include "paco_stage_args.cuh"
 
 namespace paco {
 
-struct Pass {
-    PassKernel k;
-    PassArgs a;
-    void *tw = nullptr;            // w_L^{-r}
-};
+constexpr int MAX_PASSES = 4;
+constexpr int DIRECT_LG = 20;      // passes up to K L = 2^20 keep all their factors in a table (4 MiB, 8 in FP64)
 
 struct Route {
-    int n = 0;                     // passes of paco_execute (0: the two stages)
-    Pass p[3];
-    Pass power[2];                 // the stages of the weighted power (fn == nullptr: the stage kernels)
+    int n = 0;                     // passes of paco_execute (0: the stage kernels)
+    FoldKernel k[MAX_PASSES];
+    int twmode[MAX_PASSES] = {};       // FoldCfg::TW
+    FoldArgs<float> f[MAX_PASSES];     // by the plan's precision
+    FoldArgs<double> d[MAX_PASSES];
+    PowerKernel pk[2];              // the stages of the weighted power (fn == nullptr: the stage kernels)
+    PowerArgs pa[2];
+    void *tw[MAX_PASSES + 2] = {};     // the factors of every pass, w_L^{-r} of the two stages
+    void *lo64 = nullptr, *hi64 = nullptr;
 };
 
 // pi over `bits` bits with digits of t bits (host copy of digit_reverse).
@@ -41,146 +46,251 @@ static unsigned rev_host(unsigned u, int bits, int t)
 void route_destroy(Route *r)
 {
     if (!r) return;
-    for (Pass &p : r->p) cudaFree(p.tw);
-    for (Pass &p : r->power) cudaFree(p.tw);
+    for (void *p : r->tw) cudaFree(p);
+    cudaFree(r->lo64);
+    cudaFree(r->hi64);
     delete r;
 }
 
-// Pass i of the n factors f: strides, row maps and tables.
-static paco_status_t pass_setup(const paco_plan *pl, Pass *p, const int *f, int n, int i, int t)
+// Tables of a pass's factors, each rounded once, over K = 2^lgK columns (kappa).
+enum TauKind {
+    TAU_LEVELS,     // entry q A' + k_lo: w_{K A' n}^{-(kappa + K k_lo + K A' s)}, q = tau_index(n, s), A' = 2^lgA
+    TAU_ROWS,       // entry r: w_{K A'}^{-kappa r}
+    TAU_POWERS      // entry i: w_{K A'}^{-kappa 2^i}
+};
+template <typename R>
+__global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, int lgK)
 {
-    PassArgs &a = p->a;
-    const PassKernel &k = p->k;
-    memset(&a, 0, sizeof(a));
-    int lgN = 0;
-    for (int j = 0; j < n; ++j) lgN += f[j];
-    const int lgL = f[i];
-    const int lgC = (i == 0 || i == n - 1) ? lgN - lgL : f[0];      // columns of one row block, and the row stride
-    a.bstride = pl->N;
-    a.ld_in = 1u << lgC;
-    a.ld_out = i == 0 ? 1u << lgL : 1u << lgC;
-    a.rev_bits = i == 0 ? 0 : lgL;
-    a.rev_t = t;
-    for (int j = 0; j < (1 << k.lgA); ++j) a.rowA[j] = rev_host((unsigned)j << k.lgB, a.rev_bits, t) << lgC;
-    for (int j = 0; j < (1 << k.lgB); ++j) a.rowK[j] = (unsigned)j << (k.lgA + lgC);
-    a.crev_bits = i == 0 ? lgC : (i < n - 1) ? f[2] : 0;
-    a.crev_t = t;
-    a.lg_tiles = lgC - k.lgW;
-    a.blk_stride = 1u << (f[0] + f[1]);
-    a.lg_all = lgN - lgL - k.lgW;
-    a.lo = static_cast<const cx<float> *>(pl->twN_lo);
-    a.hi = static_cast<const cx<float> *>(pl->twN_hi);
-    a.lo_bits = pl->twN_lo_bits;
-    a.tw_mul = 1u << f[0];
-    a.n_mask = (unsigned)(pl->N - 1);
-    a.mult = 1.f;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= count) return;
+    const long long kap = i & ((1ll << lgK) - 1);
+    const int q = (int)(i >> lgK);
+    long long e;
+    int lgM = lgK + lgA;
+    if (kind == TAU_LEVELS) {
+        const int klo = q & ((1 << lgA) - 1), t = q >> lgA;
+        const int lgq = t ? 31 - __clz(t) : 0, s = t ? t - (1 << lgq) : 0;
+        e = kap + ((long long)klo << lgK) + ((long long)s << lgM);
+        lgM += t ? lgq + 2 : 1;
+    } else {
+        e = kind == TAU_ROWS ? kap * q : kap << q;
+    }
+    double sn, cs;
+    sincospi(2.0 * (double)e / (double)(1ll << lgM), &sn, &cs);
+    out[i] = make_cx<R>((R)cs, (R)(-sn));
+}
+
+template <typename R>
+static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, cudaStream_t s)
+{
+    const long long count = (long long)entries << lgK;
+    tau_gen_kernel<R><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(t, count, kind, lgA, lgK);
+    return t + count;
+}
+
+// FoldArgs::tau in mode FoldCfg::TW over 2^lgK columns.
+template <typename R>
+static paco_status_t tau_table(void **dst, const FoldKernel &k, int mode, int lgK)
+{
+    const int A = 1 << k.lgA, B = 1 << k.lgB, lgL = k.lgA + k.lgB;
+    const bool fp64 = sizeof(R) == 8;
+    if (mode == 0 && fp64) return gen_table(16, dst, A * B, A * B, 1, 0);
+    const int nA = fp64 ? A : A / 2;
+    const long long cols = 1ll << lgK;
+    const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (fp64 && mode == 2 ? (nA + k.lgB) * cols : 0);
+    PACO_CUDA_TRY(cudaMalloc(dst, (size_t)count * sizeof(cx<R>)));
+    cx<R> *t = static_cast<cx<R> *>(*dst);
+    if (mode == 1) {
+        t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, 0) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, 0);
+        tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, 0);
+    } else {
+        t = tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, 0, 0);
+        if (fp64 && mode == 2) {
+            t = tau_gen(t, A, TAU_ROWS, k.lgA, lgK, 0);
+            tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK, 0);
+        }
+    }
+    PACO_CUDA_TRY(cudaGetLastError());
+    return PACO_OK;
+}
+
+// Pass i of the n factors f (log2): its strides, row maps and tables.  Its
+// columns are the frequencies of the passes before it (the first pass: all
+// other rows of the view).
+template <typename R>
+static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, const int *f, int n, int i, int t)
+{
+    const FoldKernel &k = r->k[i];
+    memset(a, 0, sizeof(*a));
+    int lgN = 0, lgK = 0;
+    for (int j = 0; j < n; ++j) {
+        lgN += f[j];
+        if (j < i) lgK += f[j];
+    }
+    const int lgL = f[i], lgC = i == 0 ? lgN - lgL : lgK;
+    a->bstride = pl->N;
+    a->ld_in = 1u << lgC;
+    a->ld_out = i == 0 ? 1u << lgL : 1u << lgC;
+    a->rev_bits = i == 0 ? 0 : lgL;
+    a->rev_t = t;
+    for (int j = 0; j < (1 << k.lgA); ++j) a->rowA[j] = rev_host((unsigned)j << k.lgB, a->rev_bits, t) << lgC;
+    for (int j = 0; j < (1 << k.lgB); ++j) a->rowK[j] = (unsigned)j << (k.lgA + lgC);
+    a->crev_bits = i == 0 ? lgC : 0;
+    a->crev_t = t;
+    a->lg_tiles = lgC - k.lgW;
+    a->lg_all = lgN - lgL - k.lgW;
+    a->blk_stride = i == 0 || i == n - 1 ? 0u : 1u << (lgK + lgL);
+    a->lo_bits = pl->twN_lo_bits;
+    a->lg_n = lgN;
+    a->lg_k = lgK;
+    a->mult = R(1);
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    const paco_status_t st = gen_table(8, &p->tw, 1LL << lgL, 1LL << lgL, 1, 0);
-    a.twL = static_cast<const cx<float> *>(p->tw);
+    paco_status_t st = tau_table<R>(&r->tw[i], k, r->twmode[i], lgK);
+    a->tau = static_cast<const cx<R> *>(r->tw[i]);
+    if (st != PACO_OK || r->twmode[i] != 2 || sizeof(R) == 8) return st;
+    // w_N^{-r} in FP64, two levels
+    if (!r->lo64) {
+        const long long nlo = 1LL << pl->twN_lo_bits;
+        if ((st = gen_table(16, &r->lo64, pl->N, nlo, 1, 0)) != PACO_OK ||
+            (st = gen_table(16, &r->hi64, pl->N, pl->N / nlo, nlo, 0)) != PACO_OK)
+            return st;
+    }
+    a->lo = static_cast<const cx<double> *>(r->lo64);
+    a->hi = static_cast<const cx<double> *>(r->hi64);
+    return PACO_OK;
+}
+
+// Stage i of the weighted power over the plan's factors.
+static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerKernel &k, void **tw, const int *lg, int i)
+{
+    memset(a, 0, sizeof(*a));
+    const int lgL = lg[i], lgC = lg[1 - i];
+    a->bstride = pl->N;
+    a->ld_in = 1u << lgC;
+    a->ld_out = i == 0 ? 1u << lgL : 1u << lgC;
+    a->rev_bits = i == 0 ? 0 : lgL;
+    a->rev_t = a->crev_t = pl->t;
+    for (int j = 0; j < (1 << k.lgA); ++j) a->rowA[j] = rev_host((unsigned)j << k.lgB, a->rev_bits, pl->t) << lgC;
+    for (int j = 0; j < (1 << k.lgB); ++j) a->rowK[j] = (unsigned)j << (k.lgA + lgC);
+    a->crev_bits = i == 0 ? lgC : 0;
+    a->lg_all = lgC - k.lgW;
+    a->lo = static_cast<const cx<float> *>(pl->twN_lo);
+    a->hi = static_cast<const cx<float> *>(pl->twN_hi);
+    a->lo_bits = pl->twN_lo_bits;
+    a->n_mask = (unsigned)(pl->N - 1);
+    PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
+    const paco_status_t st = gen_table(8, tw, 1LL << lgL, 1LL << lgL, 1, 0);
+    a->twL = static_cast<const cx<float> *>(*tw);
     return st;
 }
 
 // Factors of the route, log2, first pass first; returns their number (0: none).
 static int route_factors(const paco_plan *pl, int lg1, int lg2, int *f)
 {
-    if (pl->dims == 3) {
+    if (pl->dims >= 2) {
         f[0] = lg1;
-        f[1] = pl->lgLa3;
-        f[2] = lg2 - pl->lgLa3;
-        return 3;
+        f[1] = pl->dims == 3 ? pl->lgLa3 : lg2;
+        f[2] = lg2 - f[1];
+        return pl->dims;
     }
-    if (pl->dims == 2) {
-        f[0] = lg1;
-        f[1] = lg2;
-        return 2;
+    // as even as possible, the larger ones first (the first pass has no twiddles)
+    const int lg = lg1 + lg2, most = pl->esize == 8 ? 10 : 9;
+    int n = (lg + most - 1) / most;
+    if (n < 2) n = 2;
+    for (int i = 0, left = lg; i < n; ++i) {
+        f[i] = (left + n - i - 1) / (n - i);
+        left -= f[i];
     }
-    const int lg = lg1 + lg2;
-    if (lg < 10 || lg > 30) return 0;
-    if (lg <= 20) {
-        f[0] = lg / 2;
-        f[1] = lg - f[0];
-        return 2;
-    }
-    f[0] = (lg + 2) / 3;
-    f[1] = (lg - f[0] + 1) / 2;
-    f[2] = lg - f[0] - f[1];
-    return 3;
+    return n;
 }
 
-// Builds pl->route; leaves it nullptr where the stage kernels run the plan.
+// Builds pl->route; its n stays 0 where the stage kernels run the plan.
 paco_status_t route_setup(paco_plan *pl)
 {
-    // the plain complex64 form with no stage option asked for
-    if (pl->form || pl->shard_G || pl->esize != 8 || pl->req_split || pl->req_ctas || pl->req_tile) return PACO_OK;
+    // the plain forms with no stage option asked for
+    if (pl->form || pl->shard_G || pl->req_split || pl->req_ctas || pl->req_tile) return PACO_OK;
     Route *r = new (std::nothrow) Route();
     if (!r) return fail(PACO_ERR_NOMEM, "out of host memory");
     pl->route = r;                                     // freed with the plan
     const int lg[2] = {ilog2_exact(pl->N1), ilog2_exact(pl->N2)}, lgN = lg[0] + lg[1];
-    int f[3] = {0, 0, 0};
+    int f[MAX_PASSES] = {0, 0, 0, 0};
     int n = pl->fused ? 0 : route_factors(pl, lg[0], lg[1], f);
-    for (int i = 0; i < n; ++i) {
-        const int lgC = (i == 0 || i == n - 1) ? lgN - f[i] : f[0];
-        r->p[i].k = i == 0 ? pass_kernel_first(f[i], lgC) : i == n - 1 ? pass_kernel_last(f[i], lgC)
-                                                                       : pass_kernel_middle(f[i], lgC);
-        if (!r->p[i].k.fn) n = 0;
+    for (int i = 0, lgK = 0; i < n; lgK += f[i], ++i) {
+        const int lgC = i == 0 ? lgN - f[0] : lgK;
+        r->twmode[i] = i == 0 || pl->dims >= 2 ? 0 : lgK + f[i] <= DIRECT_LG ? 1 : 2;
+        r->k[i] = pl->esize == 8 ? fold_kernel_f32(i == 0, r->twmode[i], f[i], lgC)
+                                 : fold_kernel_f64(i == 0, r->twmode[i], f[i], lgC);
+        if (!r->k[i].fn) n = 0;
     }
     // pi of the redistribution: the plan's base where its digits fit the factors
     int t = pl->t;
     for (int i = 1; i < n; ++i)
         if (f[i] % t) t = 1;
     paco_status_t st = PACO_OK;
-    for (int i = 0; i < n && st == PACO_OK; ++i) st = pass_setup(pl, &r->p[i], f, n, i, t);
+    for (int i = 0; i < n && st == PACO_OK; ++i)
+        st = pl->esize == 8 ? pass_setup(pl, r, &r->f[i], f, n, i, t) : pass_setup(pl, r, &r->d[i], f, n, i, t);
     r->n = n;
-    if (pl->dims == 3) return st;
+    if (pl->dims == 3 || pl->esize != 8) return st;
     for (int i = 0; i < 2 && st == PACO_OK; ++i) {
-        r->power[i].k = i == 0 ? pass_kernel_first_stage(lg[0], lg[1]) : pass_kernel_last_loss(lg[1], lg[0]);
-        if (r->power[i].k.fn) st = pass_setup(pl, &r->power[i], lg, 2, i, pl->t);
+        r->pk[i] = power_kernel(i == 0, lg[i], lg[1 - i]);
+        if (r->pk[i].fn) st = power_setup(pl, &r->pa[i], r->pk[i], &r->tw[MAX_PASSES + i], lg, i);
     }
     return st;
 }
 
 int route_passes(const paco_plan *pl) { return pl->route ? pl->route->n : 0; }
 
-static paco_status_t launch_pass(const paco_plan *pl, const PassKernel &k, PassArgs &a, const void *in, void *out,
-                                 int dir, cudaStream_t stream)
+static paco_status_t launch(const paco_plan *pl, const void *fn, void *args, int lg_all, int threads, int smem,
+                            cudaStream_t stream)
 {
-    a.in = static_cast<const cx<float> *>(in);
-    a.out = static_cast<cx<float> *>(out);
-    a.conj = dir == 1;
-    const long long tiles = (long long)pl->batch << a.lg_all;
+    const long long tiles = (long long)pl->batch << lg_all;
     if (tiles > INT32_MAX) return fail(PACO_ERR_UNSUPPORTED, "batch of %lld transforms is too large", (long long)pl->batch);
-    void *params[] = {&a};
-    PACO_CUDA_TRY(cudaLaunchKernel(k.fn, dim3((unsigned)tiles), dim3((unsigned)k.threads), params, (size_t)k.smem,
-                                   stream));
+    void *params[] = {args};
+    PACO_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)tiles), dim3((unsigned)threads), params, (size_t)smem, stream));
+    return PACO_OK;
+}
+
+template <typename R>
+static paco_status_t run_passes(const paco_plan *pl, const FoldArgs<R> *args, const void *in, void *out, int dir,
+                                const StageTerms *terms, cudaStream_t stream)
+{
+    const Route &r = *pl->route;
+    for (int i = 0; i < r.n; ++i) {
+        FoldArgs<R> a = args[i];
+        a.in = static_cast<const cx<R> *>(i == 0 ? in : out);
+        a.out = static_cast<cx<R> *>(out);
+        a.conj = dir == 1;
+        if (terms && i == 0) {
+            a.mult = (R)terms->ld_mult;
+            a.scale = terms->ld_scale;
+        }
+        const paco_status_t st = launch(pl, r.k[i].fn, &a, a.lg_all, r.k[i].threads, r.k[i].smem, stream);
+        if (st != PACO_OK) return st;
+    }
     return PACO_OK;
 }
 
 paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir, const StageTerms *terms,
                         cudaStream_t stream)
 {
-    const Route &r = *pl->route;
-    for (int i = 0; i < r.n; ++i) {
-        PassArgs a = r.p[i].a;
-        if (terms && i == 0) {
-            a.mult = terms->ld_mult;
-            a.scale = terms->ld_scale;
-        }
-        const paco_status_t st = launch_pass(pl, r.p[i].k, a, i == 0 ? in : out, out, dir, stream);
-        if (st != PACO_OK) return st;
-    }
-    return PACO_OK;
+    return pl->esize == 8 ? run_passes(pl, pl->route->f, in, out, dir, terms, stream)
+                          : run_passes(pl, pl->route->d, in, out, dir, terms, stream);
 }
 
-bool route_has_power(const paco_plan *pl, int stage) { return pl->route && pl->route->power[stage].k.fn; }
+bool route_has_power(const paco_plan *pl, int stage) { return pl->route && pl->route->pk[stage].fn; }
 
 paco_status_t route_power(const paco_plan *pl, int stage, const void *in, void *out, int dir, const StageTerms &terms,
                           cudaStream_t stream)
 {
-    PassArgs a = pl->route->power[stage].a;
+    const PowerKernel &k = pl->route->pk[stage];
+    PowerArgs a = pl->route->pa[stage];
+    a.in = static_cast<const cx<float> *>(in);
+    a.out = static_cast<cx<float> *>(out);
+    a.conj = dir == 1;
     a.w = terms.st_w;
     a.loss = terms.st_loss;
     a.store_weighted = terms.st_weighted;
-    return launch_pass(pl, pl->route->power[stage].k, a, in, out, dir, stream);
+    return launch(pl, k.fn, &a, a.lg_all, k.threads, k.smem, stream);
 }
 
 } // namespace paco

@@ -1,4 +1,4 @@
-"""The passes of paco_execute (csrc/paco_pass.cuh, paco_route.cu): every pass
+"""The passes of paco_execute (csrc/paco_fold.cuh, paco_power.cuh, paco_route.cu): every pass
 length as first, middle and last pass, both directions, ragged batches, the 2-D
 and 3-D forms, and the passes of the weighted power, whose arithmetic is that of
 the stage kernels."""
@@ -47,6 +47,19 @@ def test_passes_against_oracle(l1, l2, b, batch, passes, d):
     x = uniform(batch * N, l1 + 31 * l2, np.complex64).reshape(batch, N)
     ref = oracle.fft(x.astype(np.complex128), dir=d, threads=0)
     assert _err(_run(plan, x, d), ref) <= 5e-7 * math.log2(N)
+
+
+@pytest.mark.parametrize("d", [-1, 1])
+@pytest.mark.parametrize("l1,l2,b,batch,passes", [
+    (5, 5, 2, 5, 2), (6, 5, 2, 5, 2), (6, 6, 8, 7, 2), (7, 7, 2, 3, 2), (9, 9, 2, 2, 2), (9, 10, 2, 2, 3), (11, 10, 2, 1, 3),
+    (12, 12, 4, 1, 3)])
+def test_double_passes_against_oracle(l1, l2, b, batch, passes, d):
+    N = 1 << (l1 + l2)
+    plan = paco.Plan(1 << l1, 1 << l2, b, batch, paco.C128)
+    assert plan.info.passes == passes
+    x = uniform(batch * N, l1 + 31 * l2, np.complex128).reshape(batch, N)
+    ref = oracle.fft(x, dir=d, threads=0)
+    assert _err(_run(plan, x, d), ref) <= 1e-14 * math.log2(N)
 
 
 @pytest.mark.parametrize("d", [-1, 1])

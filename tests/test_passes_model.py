@@ -1,9 +1,11 @@
-"""CPU model of the address maps of csrc/paco_pass.cuh / paco_route.cu: the
+"""CPU model of the address maps of csrc/paco_fold.cuh / paco_route.cu: the
 passes' row maps (a per-thread term for j_lo plus a launch constant for j_hi),
-the redistribution in the first pass's store addresses and the row blocks of
-the middle pass, composed over every column to numpy's DFT.  Each pass reads
+the redistribution in the first pass's store addresses, the row blocks of the
+later passes and the twiddles w_{K L}^{-kappa j} folded into their butterflies
+(kappa = column), composed over every column to numpy's DFT.  Each pass reads
 its whole input before it writes, which the kernel does tile by tile: the test
-also checks that a tile writes exactly the places it read."""
+also checks that a tile writes exactly the places it read.  A second test
+models one folded butterfly network with the kernel's twiddle list."""
 
 import numpy as np
 import pytest
@@ -17,42 +19,93 @@ def _rev(u, bits, t):
 
 
 @pytest.mark.parametrize("f,t,dims", [((3, 4), 1, 1), ((4, 4), 2, 1), ((4, 4), 4, 1), ((3, 3, 3), 1, 1),
-                                      ((3, 3, 3), 3, 1), ((4, 3, 2), 1, 1), ((4, 2, 4), 2, 1), ((3, 4), 1, 2),
-                                      ((2, 4, 3), 1, 3)])
+                                      ((3, 3, 3), 3, 1), ((4, 3, 2), 1, 1), ((4, 2, 4), 2, 1), ((3, 3, 2, 2), 1, 1),
+                                      ((2, 2, 2, 2), 2, 1), ((3, 4), 1, 2), ((2, 4, 3), 1, 3)])
 def test_pass_address_maps(f, t, dims):
     n, lgN = len(f), sum(f)
     N = 1 << lgN
     rng = np.random.default_rng(0)
     x = rng.normal(size=N) + 1j * rng.normal(size=N)
-    w = (lambda e: np.exp(-2j * np.pi * (e % N) / N)) if dims == 1 else (lambda e: 1.0)
-    out = None
+    out, lgK = None, 0
     for i, lgL in enumerate(f):
         L, lgB = 1 << lgL, lgL // 2
-        lgC = lgN - lgL if i in (0, n - 1) else f[0]              # columns of a row block, and the row stride
+        lgC = lgN - lgL if i == 0 else lgK                        # columns of a row block, and the row stride
         rb = 0 if i == 0 else lgL
-        row_a = [_rev(j << lgB, rb, t) << lgC if rb else (j << lgB) << lgC for j in range(1 << (lgL - lgB))]
+        row_a = [(_rev(j << lgB, rb, t) if rb else j << lgB) << lgC for j in range(1 << (lgL - lgB))]
 
         def row(j):
             lo = j & ((1 << lgB) - 1)
             return row_a[j >> lgB] + ((_rev(lo, rb, t) if rb else lo) << lgC)
 
         src, dst = (x if i == 0 else out), np.full(N, np.nan, complex)
-        for blk in range(1 if i in (0, n - 1) else 1 << (lgN - lgL - lgC)):
+        for blk in range(1 << (lgN - lgL - lgC)):
             for c in range(1 << lgC):
-                base = (blk << (f[0] + f[1]) if blk else 0) + c
+                base = (blk << (lgK + lgL)) + c
                 read = [base + row(j) for j in range(L)]
-                y = np.fft.fft(src[read])
+                tw = np.exp(-2j * np.pi * c * np.arange(L) / (L << lgK)) if i > 0 and dims == 1 else 1.0
+                y = np.fft.fft(src[read] * tw)
                 for k in range(L):
-                    if i == 0:
-                        v, a = y[k] * w(k * c), _rev(c, lgC, t) * L + k
-                    else:
-                        v, a = y[k], base + (k << lgC)
-                        if i < n - 1:
-                            v = v * w(k * _rev(blk, f[2], t) << f[0])
+                    a = _rev(c, lgC, t) * L + k if i == 0 else base + (k << lgC)
                     assert np.isnan(dst[a].real)
-                    dst[a] = v
+                    dst[a] = y[k]
                 if i > 0:
                     assert sorted(read) == sorted(base + (k << lgC) for k in range(L))
-        out = dst
+        out, lgK = dst, lgK + lgL
     ref = np.fft.fft(x) if dims == 1 else np.fft.fftn(x.reshape([1 << q for q in f])).transpose(range(n)[::-1]).reshape(-1)
     assert np.max(np.abs(out - ref)) <= 1e-13 * np.max(np.abs(ref)) * lgN
+
+
+def _fold(v, tau):
+    """fold_dft: bit-reversed input, levels n = 2, 4, .., with one twiddle per
+    pair of butterflies (the second one of the pair takes -i times it)."""
+    R = len(v)
+    lg = R.bit_length() - 1
+    u = [v[_rev(i, lg, 1)] for i in range(R)]
+    n = 2
+    while n <= R:
+        q = max(1, n // 4)
+        for s in range(q):
+            for b in range(0, R, n):
+                for off, t in [(s, tau(n, s))] + ([(s + q, -1j * tau(n, s))] if n >= 4 else []):
+                    e, o = u[b + off], t * u[b + off + n // 2]
+                    u[b + off], u[b + off + n // 2] = e + o, e - o
+        n *= 2
+    return np.array(u)
+
+
+@pytest.mark.parametrize("lgA,lgB,lgK,lgN", [(4, 1, 6, 11), (3, 3, 5, 12), (4, 3, 7, 14), (5, 4, 3, 15), (5, 5, 2, 12)])
+def test_folded_twiddles(lgA, lgB, lgK, lgN):
+    """Both halves of a pass: the columns' list (as the kernel inverts its
+    index), w_{K L}^{-kappa 2^i} times w_L^{-(k_lo + s A) 2^i}, and the result."""
+    A, B, K, N = 1 << lgA, 1 << lgB, 1 << lgK, 1 << lgN
+    L = A * B
+    w = lambda m, e: np.exp(-2j * np.pi * e / m)  # noqa: E731
+    rng = np.random.default_rng(1)
+    for kap in {0, 1, K // 2, K - 1}:
+        x = rng.normal(size=L) + 1j * rng.normal(size=L)
+        lst, sizes = [], []
+        for i in range(max(1, A // 2)):
+            left = A // 2 - 1 - i
+            lgq = left.bit_length() - 1 if left else 0
+            lgn, s = (lgq + 2, (2 << lgq) - 1 - left) if left else (1, 0)
+            e = ((kap + (s << lgK)) << (lgA - lgn)) << (lgN - lgK - lgA)
+            assert 0 <= e < N
+            lst.append(w(N, e))
+            sizes.append((1 << lgn, s))
+        index = {}
+        n, i = A, 0
+        while n >= 2:
+            for s in range(max(1, n // 4)):
+                index[n, s] = i
+                i += 1
+            n //= 2
+        assert [index[z] for z in sizes] == list(range(len(sizes)))
+        F1 = np.array([_fold([x[r * B + jlo] for r in range(A)], lambda n, s: lst[index[n, s]]) for jlo in range(B)])
+        y = np.empty(L, complex)
+        for klo in range(A):
+            def tau(n, s):
+                lg = (B // n).bit_length() - 1
+                return w(L, (klo + s * A) * (B // n)) * w(N, (kap << lg) << (lgN - lgK - lgA - lgB))
+            y[klo + A * np.arange(B)] = _fold(list(F1[:, klo]), tau)
+        ref = np.fft.fft(x * w(K * L, kap * np.arange(L)))
+        assert np.max(np.abs(y - ref)) <= 1e-12 * np.max(np.abs(ref))
