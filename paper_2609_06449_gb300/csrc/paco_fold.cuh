@@ -210,8 +210,10 @@ struct FoldCfg {
     static constexpr int MINB = REGS_CTAS < 1 ? 1 : (REGS_CTAS < SMEM_CTAS ? REGS_CTAS : SMEM_CTAS);
 };
 
+// One tile of the transform at element offset boff.
 template <class CFG>
-__global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __grid_constant__ FoldArgs<typename CFG::R> a)
+__device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, int tile, long long boff,
+                                          unsigned char *smem_raw)
 {
     using R = typename CFG::R;
     using C = cx<R>;
@@ -219,13 +221,10 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __g
     constexpr int A = CFG::A, B = CFG::B, W = CFG::W, NT = CFG::NT, U1 = CFG::U1, U2 = CFG::U2;
     constexpr bool FIRST = CFG::FIRST;
     constexpr int TW = CFG::TW;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     C *sm = reinterpret_cast<C *>(smem_raw);
     [[maybe_unused]] C *tabA = sm + CFG::EX;       // TW 2: [tau index][col]
     [[maybe_unused]] C *tabB = tabA + CFG::NA * W; //       [i][col]: w_{K L}^{-kappa 2^i}
     const int tid = threadIdx.x;
-    const int tile = (int)(blockIdx.x & ((1u << a.lg_all) - 1u));
-    const long long boff = (long long)(blockIdx.x >> a.lg_all) * a.bstride;
     const int blk = FIRST ? 0 : tile >> a.lg_tiles;
     const unsigned c0 = (unsigned)(FIRST ? tile : tile & ((1 << a.lg_tiles) - 1)) << CFG::LGW;
     const long long base = boff + (long long)blk * (FIRST ? 0u : a.blk_stride) + c0;
@@ -373,6 +372,13 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __g
             q[FIRST ? (unsigned)(A * k) : a.rowK[k]] = o;
         }
     }
+}
+
+template <class CFG>
+__global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __grid_constant__ FoldArgs<typename CFG::R> a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fold_tile<CFG>(a, (int)(blockIdx.x & ((1u << a.lg_all) - 1u)), (long long)(blockIdx.x >> a.lg_all) * a.bstride, smem_raw);
 }
 
 // What the host needs to launch one of the kernels above.

@@ -19,6 +19,7 @@
 #include "paco_power.cuh"
 #include "paco_plan.h"
 #include "paco_stage_args.cuh"
+#include "paco_whole.cuh"
 
 namespace paco {
 
@@ -27,6 +28,7 @@ constexpr int DIRECT_LG = 20;      // passes up to K L = 2^20 keep all their fac
 
 struct Route {
     int n = 0;                     // passes of paco_execute (0: the stage kernels)
+    WholeKernel whole;             // n = 1: whole transforms in a CTA
     FoldKernel k[MAX_PASSES];
     int twmode[MAX_PASSES] = {};       // FoldCfg::TW
     FoldArgs<float> f[MAX_PASSES];     // by the plan's precision
@@ -110,6 +112,19 @@ static paco_status_t tau_table(void **dst, const FoldKernel &k, int mode, int lg
             tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK, 0);
         }
     }
+    PACO_CUDA_TRY(cudaGetLastError());
+    return PACO_OK;
+}
+
+paco_status_t whole_table(int lgN, void **dst)
+{
+    int k[4], n = 0, total = 0;                            // log2 of the frequencies known before every step
+    k[0] = 0;
+    for (; n < 3 && whole_radix(lgN, n); ++n) k[n + 1] = k[n] + ilog2_exact(whole_radix(lgN, n));
+    for (int i = 1; i < n; ++i) total += 1 << (k[i + 1] - 1);
+    PACO_CUDA_TRY(cudaMalloc(dst, (size_t)total * 8));
+    cx<float> *t = static_cast<cx<float> *>(*dst);
+    for (int i = 1; i < n; ++i) t = tau_gen(t, 1 << (k[i + 1] - 1), TAU_LEVELS, k[i], 0, 0);
     PACO_CUDA_TRY(cudaGetLastError());
     return PACO_OK;
 }
@@ -214,7 +229,14 @@ paco_status_t route_setup(paco_plan *pl)
     pl->route = r;                                     // freed with the plan
     const int lg[2] = {ilog2_exact(pl->N1), ilog2_exact(pl->N2)}, lgN = lg[0] + lg[1];
     int f[MAX_PASSES] = {0, 0, 0, 0};
-    int n = pl->fused ? 0 : route_factors(pl, lg[0], lg[1], f);
+    // short transforms: one CTA holds them whole
+    if (pl->dims == 1 && pl->esize == 8 && (r->whole = whole_kernel(lgN)).fn) {
+        const paco_status_t st = whole_table(lgN, &r->tw[0]);
+        if (st != PACO_OK) return st;
+        PACO_CUDA_TRY(cudaFuncSetAttribute(r->whole.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->whole.smem));
+        r->n = 1;
+    }
+    int n = pl->fused || r->n ? 0 : route_factors(pl, lg[0], lg[1], f);
     for (int i = 0, lgK = 0; i < n; lgK += f[i], ++i) {
         const int lgC = i == 0 ? lgN - f[0] : lgK;
         r->twmode[i] = i == 0 || pl->dims >= 2 ? 0 : lgK + f[i] <= DIRECT_LG ? 1 : 2;
@@ -229,7 +251,7 @@ paco_status_t route_setup(paco_plan *pl)
     paco_status_t st = PACO_OK;
     for (int i = 0; i < n && st == PACO_OK; ++i)
         st = pl->esize == 8 ? pass_setup(pl, r, &r->f[i], f, n, i, t) : pass_setup(pl, r, &r->d[i], f, n, i, t);
-    r->n = n;
+    if (n) r->n = n;
     if (pl->dims == 3 || pl->esize != 8) return st;
     for (int i = 0; i < 2 && st == PACO_OK; ++i) {
         r->pk[i] = power_kernel(i == 0, lg[i], lg[1 - i]);
@@ -273,6 +295,22 @@ static paco_status_t run_passes(const paco_plan *pl, const FoldArgs<R> *args, co
 paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir, const StageTerms *terms,
                         cudaStream_t stream)
 {
+    const Route &r = *pl->route;
+    if (r.whole.fn) {
+        WholeArgs a;
+        a.in = static_cast<const float2 *>(in);
+        a.out = static_cast<float2 *>(out);
+        a.batch = pl->batch;
+        a.tau = static_cast<const float2 *>(r.tw[0]);
+        a.conj = dir == 1;
+        a.mult = terms ? terms->ld_mult : 1.f;
+        a.scale = terms ? terms->ld_scale : nullptr;
+        void *params[] = {&a};
+        const long long ctas = (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta;
+        PACO_CUDA_TRY(cudaLaunchKernel(r.whole.fn, dim3((unsigned)ctas), dim3((unsigned)r.whole.threads), params,
+                                       (size_t)r.whole.smem, stream));
+        return PACO_OK;
+    }
     return pl->esize == 8 ? run_passes(pl, pl->route->f, in, out, dir, terms, stream)
                           : run_passes(pl, pl->route->d, in, out, dir, terms, stream);
 }

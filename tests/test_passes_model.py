@@ -109,3 +109,54 @@ def test_folded_twiddles(lgA, lgB, lgK, lgN):
             y[klo + A * np.arange(B)] = _fold(list(F1[:, klo]), tau)
         ref = np.fft.fft(x * w(K * L, kap * np.arange(L)))
         assert np.max(np.abs(y - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("lg", range(4, 15))
+def test_whole_transform_exchanges(lg):
+    """paco_whole.cuh: the chain of register steps and exchanges -- every place
+    in bounds and written once, at most two points of a half-warp in one bank
+    (one from 2^6 points on, 2^9 aside), and the DFT as the result."""
+    table = [[4, 4], [8, 4], [8, 8], [8, 16], [16, 16], [8, 8, 8], [16, 8, 8], [16, 16, 8], [16, 16, 16],
+             [32, 16, 16], [32, 32, 16]]
+    R, N = table[lg - 4], 1 << lg
+    ept, nt = (16, 256) if lg <= 12 else (32, 256) if lg == 13 else (32, 512)
+    G, K = ept * nt // N, [1]
+    for r in R:
+        K.append(K[-1] * r)
+
+    def gs(i):
+        b = N // K[i + 1] * (K[i + 1] + 1)
+        return (b + 7) // 16 * 16 + 8 if K[i + 1] < 16 else b
+
+    size = max(G * gs(i) for i in range(len(R) - 1))
+    assert size * 8 <= 227 * 1024
+    rng = np.random.default_rng(0)
+    x = rng.normal(size=(G, N)) + 1j * rng.normal(size=(G, N))
+    buf, out, conflicts = None, np.full((G, N), np.nan, complex), 0
+
+    def banks(ad):
+        return max(int(np.bincount(ad[h:h + 16, 0] % 16).max()) for h in range(0, len(ad), 16))
+
+    for i, r in enumerate(R):
+        sq, j = N // r, N // r // K[i]
+        s, rr = np.arange(G * N // r), np.arange(r)
+        g, idx = s // sq, s % sq
+        kap, jlo = idx % K[i], idx // K[i]
+        if i == 0:
+            v = x[g[:, None], idx[:, None] + rr * sq]
+        else:
+            ad = (g * gs(i - 1) + kap + (K[i] + 1) * jlo)[:, None] + (K[i] + 1) * j * rr
+            conflicts = max(conflicts, banks(ad))
+            v = buf[ad]
+        y = np.fft.fft(v * np.exp(-2j * np.pi * kap[:, None] * rr / (K[i] * r)), axis=1)
+        if i < len(R) - 1:
+            ad = (g * gs(i) + kap + (K[i] * r + 1) * jlo)[:, None] + K[i] * rr
+            assert ad.max() < size and len(np.unique(ad)) == ad.size
+            conflicts = max(conflicts, banks(ad))
+            buf = np.full(size, np.nan, complex)
+            buf[ad] = y
+        else:
+            out[g[:, None], kap[:, None] + K[i] * rr] = y
+    ref = np.fft.fft(x, axis=1)
+    assert np.max(np.abs(out - ref)) <= 1e-13 * np.max(np.abs(ref))
+    assert conflicts <= (1 if lg >= 6 and lg != 9 else 2)
