@@ -10,24 +10,21 @@
 // one queue of equal-sized work items (8192 elements each), claimed in order
 // by a persistent grid.
 //
-//   small item  (N <= 2^13): G = 8192 / N whole transforms in one CTA.  Both
-//               local FFTs run in shared memory; the redistribution is an
-//               index map inside the CTA (self pairs only), so the transform
-//               costs one HBM read and one HBM write per element.
-//   stage item  (N >= 2^14): one tile of Phase I (mode 1) or Phase III
-//               (mode 2) of one transform, the stage_tile body of the
-//               single-length kernels with a tile of L x (8192 / L).  A
-//               Phase III tile waits (bounded) on the transform's counter of
-//               finished Phase I tiles.  Items are ordered so that a
-//               transform's Phase III comes a fixed lag after its Phase I,
-//               long enough to avoid waiting and short enough for W to stay
-//               in L2 between the two (at best 16 B of HBM traffic per
-//               element instead of 32).
+//   small item  (N <= 2^13): G = 8192 / N whole transforms in one CTA
+//               (paco_whole.cuh): one HBM read and one HBM write per element.
+//   stage item  (N >= 2^14): one tile (8192 elements) of Phase I (kind 1) or
+//               Phase III (kind 2) of one transform, the pass of paco_fold.cuh
+//               that paco_execute runs for a single length.  A Phase III tile
+//               waits (bounded) on the transform's counter of finished Phase I
+//               tiles.  Items are ordered so that a transform's Phase III comes
+//               a fixed lag after its Phase I, long enough to avoid waiting and
+//               short enough for W to stay in L2 between the two (at best 16 B
+//               of HBM traffic per element instead of 32).
 //
-// The plan's autotuner picks, per length, the N1 x N2 split and the radix b,
-// and for the whole batch the kernel variant (one or two CTAs per SM) and the
-// lag, by timing candidates at plan creation; it optimises time, so part of
-// the L2 residency can be traded for faster tiles.
+// The plan's autotuner picks, per length, the N1 x N2 split and, for the whole
+// batch, the CTAs per SM and the lag, by timing candidates at plan creation;
+// the radix b of the redistribution is the largest that both factors are powers
+// of (its index maps cost the same for every b).
 //
 // Deadlock freedom: only Phase III items wait, and only on Phase I items of
 // a lower queue index; those were claimed by running CTAs and never wait, so
@@ -42,14 +39,16 @@
 #include <vector>
 
 #include "paco_common.cuh"
+#include "paco_fold.cuh"
 #include "paco_plan.h"
-#include "paco_stage.cuh"
+#include "paco_whole.cuh"
 
 namespace paco {
 
 namespace batched {
-constexpr int NT = 512;            // threads per CTA
-constexpr int ITEM = 8192;         // elements per work item
+constexpr int NT = 256;            // threads per CTA
+constexpr int EPT = 32;            // elements a thread holds
+constexpr int ITEM = NT * EPT;     // elements per work item
 constexpr int SMALL_MAX_LG = 13;   // whole-transform items up to 2^13
 constexpr int STAGE_MIN_LG = 6;    // stage lengths built: 2^6 .. 2^10
 constexpr int STAGE_MAX_LG = 10;
@@ -61,8 +60,8 @@ struct BLen {
     int small;                     // 1: whole-transform items
     int G;                         // small: transforms per item
     int ntiles1, ntiles2;          // stage items per transform
-    const void *twN;               // small: w_N^{-r}, r < N
-    StageArgs s1, s2;              // stage: mode 1 and mode 2 (in/out/conj set per item)
+    const float2 *tau;             // small: the steps' factors
+    FoldArgs<float> s1, s2;        // stage: Phase I and Phase III (in/out/conj set per item)
 };
 
 struct __align__(16) BItem {
@@ -96,276 +95,62 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
     return v;
 }
 
-// ---- whole transforms in shared memory ------------------------------------
-// S holds G transforms (natural order) of N elements.  W of transform g is
-// stored at S + g*N as rows of N1 with the columns XOR-swizzled by
-// h(row) = pi_m2(row) mod min(N1, 32) (conflict-free Phase I stores and
-// Phase III loads; any per-row bijection of the columns is a valid layout).
-template <int LG1, int LG2>
-__device__ __forceinline__ void small_group(const BatchedArgs &a, const BLen &ld, int gstart, int gcount,
-                                            cx<float> *S, long long *s_off)
-{
-    using C = cx<float>;
-    constexpr int N1 = 1 << LG1, N2 = 1 << LG2, LGN = LG1 + LG2, N = 1 << LGN;
-    constexpr int G = batched::ITEM / N;
-    constexpr int R1 = N1 < 16 ? N1 : 16, R2 = N1 / R1;        // Phase I radices
-    constexpr int Q1 = N2 < 16 ? N2 : 16, Q2 = N2 / Q1;        // Phase III radices
-    constexpr int LR1 = ilog2c<R1>::value, LR2 = ilog2c<R2>::value;
-    constexpr int LQ1 = ilog2c<Q1>::value, LQ2 = ilog2c<Q2>::value;
-    constexpr int HM = (N1 < 32 ? N1 : 32) - 1;                 // swizzle mask
-    const int tid = threadIdx.x;
-    const int t = ld.t;
-    const bool cj = a.conj != 0;
-    // w_N^{-r} = lo[r mod 2^LH] * hi[r >> LH], both halves in shared memory
-    constexpr int LH = (LGN + 1) / 2;
-    C *tw_lo = reinterpret_cast<C *>(s_off + G);
-    C *tw_hi = tw_lo + (1 << LH);
-    {
-        const C *tw = reinterpret_cast<const C *>(ld.twN);
-        for (int r = tid; r < (1 << LH); r += batched::NT) tw_lo[r] = tw[r];
-        for (int r = tid; r < (N >> LH); r += batched::NT) tw_hi[r] = tw[r << LH];
-    }
-    auto twid = [&](int r) { return cmul(tw_lo[r & ((1 << LH) - 1)], tw_hi[r >> LH]); };
-    // z^s, s < 16, for z = w_N^{-e}: from z, z^4, z^8 (three table reads)
-    // and at most two products, zh[s >> 2] * zl[s & 3]
-    auto powers = [&](C (&zl)[4], C (&zh)[4], int e) {
-        const C z1 = twid(e & (N - 1)), z4 = twid((4 * e) & (N - 1)), z8 = twid((8 * e) & (N - 1));
-        zl[0] = make_cx<float>(1.f, 0.f); zl[1] = z1; zl[2] = cmul(z1, z1); zl[3] = cmul(zl[2], z1);
-        zh[0] = make_cx<float>(1.f, 0.f); zh[1] = z4; zh[2] = z8; zh[3] = cmul(z8, z4);
-    };
-    auto zpow = [&](const C (&zl)[4], const C (&zh)[4], int s_) {
-        return ((s_ & 3) == 0) ? zh[s_ >> 2] : ((s_ >> 2) == 0) ? zl[s_ & 3] : cmul(zh[s_ >> 2], zl[s_ & 3]);
-    };
+// Tiles of a stage of length 2^LG: factors A B and columns, 8192 elements.
+template <int LG, bool FIRST>
+using StageCfgB = FoldCfg<float, LG == 9 || LG == 10 ? 5 : LG == 6 ? 3 : 4, LG == 10 ? 5 : LG >= 8 ? 4 : 3, 13 - LG, FIRST,
+                          1, batched::EPT>;
 
-    for (int g = tid; g < gcount; g += batched::NT) s_off[g] = a.off[a.group_tx[gstart + g]];
-    __syncthreads();
-    // load: 16-byte vectors, all issued before any use, conjugated for dir = +1
-    {
-        constexpr int NV = batched::ITEM / 2 / batched::NT;
-        const float4 *src = reinterpret_cast<const float4 *>(a.in);
-        float4 r4[NV];
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = tid + batched::NT * i;
-            const int g = (2 * e) >> LGN, r = (2 * e) & (N - 1);
-            r4[i] = (g < gcount) ? __ldg(src + ((s_off[g] + r) >> 1)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = tid + batched::NT * i;
-            float4 v4 = r4[i];
-            if (cj) { v4.y = -v4.y; v4.w = -v4.w; }
-            S[2 * e] = make_cx<float>(v4.x, v4.y);
-            S[2 * e + 1] = make_cx<float>(v4.z, v4.w);
-        }
-    }
-    __syncthreads();
-
-    C v[16];
-    // ---- Phase I pass a: radix R1 over j_hi (j = j_hi*R2 + j_lo), twiddle
-    //      w_N1^{-k_lo j_lo}, back in place (k_lo*R2 + j_lo)
-    constexpr int NUa = 16 / R1;
-#pragma unroll
-    for (int q = 0; q < NUa; ++q) {
-        const int u = tid + batched::NT * q;
-        const int c = u & (N2 - 1);
-        const int jl = (u >> LG2) & (R2 - 1);
-        const int g = u >> (LG2 + LR2);
-        C *base = S + g * N + jl * N2 + c;
-#pragma unroll
-        for (int r = 0; r < R1; ++r) v[q * R1 + r] = base[r * R2 * N2];
-        dft<R1>(v + q * R1);
-        if constexpr (R2 > 1) {
-            C zl[4], zh[4];
-            powers(zl, zh, jl * N2);                           // w_N1^{-jl} = w_N^{-jl N2}
-#pragma unroll
-            for (int s = 1; s < R1; ++s) v[q * R1 + s] = cmul(v[q * R1 + s], zpow(zl, zh, s));
-#pragma unroll
-            for (int s = 0; s < R1; ++s) base[s * R2 * N2] = v[q * R1 + s];
-        }
-    }
-    // ---- Phase I pass b: radix R2 over j_lo; k1 = k_lo + R1 * k_hi
-    constexpr int NUb = 16 / R2;
-    if constexpr (R2 > 1) {
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < NUb; ++q) {
-            const int u = tid + batched::NT * q;
-            const int c = u & (N2 - 1);
-            const int kl = (u >> LG2) & (R1 - 1);
-            const int g = u >> (LG2 + LR1);
-            const C *base = S + g * N + kl * R2 * N2 + c;
-#pragma unroll
-            for (int r = 0; r < R2; ++r) v[q * R2 + r] = base[r * N2];
-            dft<R2>(v + q * R2);
-        }
-    }
-    __syncthreads();        // every Phase I read done before W overwrites S
-    // ---- top-level twiddle w_N^{-k1 c} and the fused digit reversal:
-    //      Z[k1][c] -> W[pi_m2(c)][k1]
-    {
-        constexpr int NUf = (R2 > 1) ? NUb : NUa;
-        constexpr int RF = (R2 > 1) ? R2 : R1;
-#pragma unroll
-        for (int q = 0; q < NUf; ++q) {
-            const int u = tid + batched::NT * q;
-            const int c = u & (N2 - 1);
-            const int kl = (R2 > 1) ? ((u >> LG2) & (R1 - 1)) : 0;
-            const int g = (R2 > 1) ? (u >> (LG2 + LR1)) : (u >> LG2);
-            const int urow = (int)digit_reverse((unsigned)c, LG2, t);
-            C *row = S + g * N + urow * N1;
-            const int h = c & HM;                              // pi_m2(urow) = c
-#pragma unroll
-            for (int k = 0; k < RF; ++k) {
-                const int k1 = (R2 > 1) ? (kl + R1 * k) : k;
-                row[k1 ^ h] = cmul(v[q * RF + k], twid(k1 * c));
-            }
-        }
-    }
-    __syncthreads();
-    // ---- Phase III pass a: column v of W through the row map j -> pi_m2(j);
-    //      radix Q1 over j_hi (j = j_hi*Q2 + j_lo), twiddle w_N2^{-k_lo j_lo}
-    constexpr int NUc = 16 / Q1;
-    constexpr int NUd = 16 / Q2;
-    C *gout = reinterpret_cast<C *>(a.out);
-#pragma unroll
-    for (int q = 0; q < NUc; ++q) {
-        const int u = tid + batched::NT * q;
-        const int col = u & (N1 - 1);
-        const int jl = (u >> LG1) & (Q2 - 1);
-        const int g = u >> (LG1 + LQ2);
-        C *base = S + g * N;
-#pragma unroll
-        for (int r = 0; r < Q1; ++r) {
-            const int j = r * Q2 + jl;
-            const int row = (int)digit_reverse((unsigned)j, LG2, t);
-            v[q * Q1 + r] = base[row * N1 + (col ^ (j & HM))];
-        }
-        dft<Q1>(v + q * Q1);
-        if constexpr (Q2 > 1) {
-            C zl[4], zh[4];
-            powers(zl, zh, jl * N1);                           // w_N2^{-jl} = w_N^{-jl N1}
-#pragma unroll
-            for (int s = 0; s < Q1; ++s) {
-                C y = (s > 0) ? cmul(v[q * Q1 + s], zpow(zl, zh, s)) : v[q * Q1 + s];
-                const int j = s * Q2 + jl;
-                const int row = (int)digit_reverse((unsigned)j, LG2, t);
-                base[row * N1 + (col ^ (j & HM))] = y;
-            }
-        } else if (g < gcount) {
-            // single pass: k2 = s, natural-order y[k2 * N1 + col]
-            C *dst = gout + s_off[g];
-#pragma unroll
-            for (int s = 0; s < Q1; ++s) {
-                C y = v[q * Q1 + s];
-                if (cj) y.y = -y.y;
-                dst[s * N1 + col] = y;
-            }
-        }
-    }
-    if constexpr (Q2 > 1) {
-        __syncthreads();
-        // ---- Phase III pass b: radix Q2 over j_lo; k2 = k_lo + Q1 * k_hi
-#pragma unroll
-        for (int q = 0; q < NUd; ++q) {
-            const int u = tid + batched::NT * q;
-            const int col = u & (N1 - 1);
-            const int kl = (u >> LG1) & (Q1 - 1);
-            const int g = u >> (LG1 + LQ1);
-            const C *base = S + g * N;
-#pragma unroll
-            for (int r = 0; r < Q2; ++r) {
-                const int j = kl * Q2 + r;
-                const int row = (int)digit_reverse((unsigned)j, LG2, t);
-                v[q * Q2 + r] = base[row * N1 + (col ^ (j & HM))];
-            }
-            dft<Q2>(v + q * Q2);
-            if (g < gcount) {
-                C *dst = gout + s_off[g];
-#pragma unroll
-                for (int k = 0; k < Q2; ++k) {
-                    C y = v[q * Q2 + k];
-                    if (cj) y.y = -y.y;
-                    dst[(kl + Q1 * k) * N1 + col] = y;
-                }
-            }
-        }
-    }
-}
-
-template <int LG1, int LG2>
-__device__ __noinline__ void small_item(const BatchedArgs &a, const BLen &ld, int gs, int gc, cx<float> *S,
-                                       long long *so)
-{
-    small_group<LG1, LG2>(a, ld, gs, gc, S, so);
-}
-
-// LDCG: Phase III reads W, written by other CTAs of this launch, through L2
-// only; Phase I reads the launch's read-only input through the read-only path.
-// One CTA per SM (128 registers): the body is inlined with the descriptor
-// taken by value, so its fields live in registers instead of being re-read
-// from shared memory after every barrier of the tile (measured ~20% faster
-// per tile).  Two CTAs per SM (64 registers): inlining spills, so the body is
-// a call.
-template <int A, int B, bool LDCG>
-__device__ __forceinline__ void stage_item_inline(const StageArgs sa, int tile, long long boff,
-                                                  unsigned char *smem)
-{
-    stage_tile<float, A, B, -1, 0, 0, LDCG>(sa, tile, boff, 0, smem);
-}
-template <int A, int B, bool LDCG>
-__device__ __noinline__ void stage_item_call(const StageArgs &sa, int tile, long long boff, unsigned char *smem)
-{
-    stage_tile<float, A, B, -1, 0, 0, LDCG>(sa, tile, boff, 0, smem);
-}
-template <int MINB, int A, int B, bool LDCG>
-__device__ __forceinline__ void stage_item(const StageArgs &sa, int tile, long long boff, unsigned char *smem)
-{
-    if constexpr (MINB == 1) stage_item_inline<A, B, LDCG>(sa, tile, boff, smem);
-    else stage_item_call<A, B, LDCG>(sa, tile, boff, smem);
-}
-
-__device__ __forceinline__ void small_dispatch(const BatchedArgs &a, const BLen &ld, int gs, int gc,
-                                               cx<float> *S, long long *so)
-{
-    switch (ld.lgN) {
-    case 4: small_item<2, 2>(a, ld, gs, gc, S, so); break;
-    case 5: small_item<3, 2>(a, ld, gs, gc, S, so); break;
-    case 6: small_item<3, 3>(a, ld, gs, gc, S, so); break;
-    case 7: small_item<4, 3>(a, ld, gs, gc, S, so); break;
-    case 8: small_item<4, 4>(a, ld, gs, gc, S, so); break;
-    case 9: small_item<5, 4>(a, ld, gs, gc, S, so); break;
-    case 10: small_item<5, 5>(a, ld, gs, gc, S, so); break;
-    case 11: small_item<6, 5>(a, ld, gs, gc, S, so); break;
-    case 12: small_item<6, 6>(a, ld, gs, gc, S, so); break;
-    case 13: small_item<7, 6>(a, ld, gs, gc, S, so); break;
-    default: break;
-    }
-}
-
-template <int MINB, bool LDCG>
-__device__ __forceinline__ void stage_dispatch(const StageArgs &sa, int lgL, int tile, long long boff,
-                                               unsigned char *smem)
+template <bool FIRST>
+__device__ __forceinline__ void stage_item(const FoldArgs<float> &sa, int lgL, int tile, long long boff, unsigned char *smem)
 {
     switch (lgL) {
-    case 6: stage_item<MINB, 8, 8, LDCG>(sa, tile, boff, smem); break;
-    case 7: stage_item<MINB, 16, 8, LDCG>(sa, tile, boff, smem); break;
-    case 8: stage_item<MINB, 16, 16, LDCG>(sa, tile, boff, smem); break;
-    case 9: stage_item<MINB, 32, 16, LDCG>(sa, tile, boff, smem); break;
-    case 10: stage_item<MINB, 32, 32, LDCG>(sa, tile, boff, smem); break;
+    case 6: fold_tile<StageCfgB<6, FIRST>>(sa, tile, boff, smem); break;
+    case 7: fold_tile<StageCfgB<7, FIRST>>(sa, tile, boff, smem); break;
+    case 8: fold_tile<StageCfgB<8, FIRST>>(sa, tile, boff, smem); break;
+    case 9: fold_tile<StageCfgB<9, FIRST>>(sa, tile, boff, smem); break;
+    case 10: fold_tile<StageCfgB<10, FIRST>>(sa, tile, boff, smem); break;
     default: break;
     }
 }
 
-template <int MINB>
-__global__ void __launch_bounds__(batched::NT, MINB) paco_batched_kernel(const __grid_constant__ BatchedArgs a)
+template <int LG>
+__device__ __forceinline__ void small_item(const BatchedArgs &a, const float2 *tau, int count, const long long *s_off,
+                                           unsigned char *smem)
+{
+    whole_step<WholeCfg<LG, batched::EPT, batched::NT>, batched::EPT, batched::NT, 0>(
+        static_cast<const float2 *>(a.in), static_cast<float2 *>(a.out), a.conj != 0, 1.f, tau,
+        [&](int g) { return g < count ? s_off[g] : -1ll; }, reinterpret_cast<cx<float> *>(smem));
+}
+
+__device__ __forceinline__ void small_dispatch(const BatchedArgs &a, int lgN, const float2 *tau, int count,
+                                               const long long *s_off, unsigned char *smem)
+{
+    switch (lgN) {
+    case 4: small_item<4>(a, tau, count, s_off, smem); break;
+    case 5: small_item<5>(a, tau, count, s_off, smem); break;
+    case 6: small_item<6>(a, tau, count, s_off, smem); break;
+    case 7: small_item<7>(a, tau, count, s_off, smem); break;
+    case 8: small_item<8>(a, tau, count, s_off, smem); break;
+    case 9: small_item<9>(a, tau, count, s_off, smem); break;
+    case 10: small_item<10>(a, tau, count, s_off, smem); break;
+    case 11: small_item<11>(a, tau, count, s_off, smem); break;
+    case 12: small_item<12>(a, tau, count, s_off, smem); break;
+    case 13: small_item<13>(a, tau, count, s_off, smem); break;
+    default: break;
+    }
+}
+
+// Two CTAs of 256 threads with 128 registers an SM (32 elements a thread: the
+// folded radix-32 steps).
+__global__ void __launch_bounds__(batched::NT, 2) paco_batched_kernel(const __grid_constant__ BatchedArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BItem s_it;
     __shared__ int s_ok;
-    __shared__ int s_key;                         // (length, kind) whose descriptor s_sa holds
-    __shared__ StageArgs s_sa;
+    __shared__ FoldArgs<float> s_sa;
+    __shared__ long long s_off[batched::ITEM / 16];   // a small group's element offsets
     const int tid = threadIdx.x;
+    int key = -1;                                 // (length, kind) whose descriptor s_sa holds
     // Thread 0 keeps the next item (claimed and loaded) and the index of the
     // one after it (claimed) in registers: both round trips overlap the
     // current item.  Claiming ahead cannot deadlock: the lowest-indexed
@@ -374,7 +159,6 @@ __global__ void __launch_bounds__(batched::NT, MINB) paco_batched_kernel(const _
     BItem nit;
     int nidx = 0, nidx2 = 0;
     if (tid == 0) {
-        s_key = -1;
         nidx = (int)atomicAdd(&a.ctr[0], 1u);
         nidx2 = (int)atomicAdd(&a.ctr[0], 1u);
         if (nidx < a.nitems) nit = a.items[nidx];
@@ -397,21 +181,23 @@ __global__ void __launch_bounds__(batched::NT, MINB) paco_batched_kernel(const _
         if (item.kind < 0) break;
         const BLen &ld = a.lens[item.len];
         if (item.kind == 0) {
-            cx<float> *S = reinterpret_cast<cx<float> *>(smem_raw);
-            long long *so = reinterpret_cast<long long *>(smem_raw + batched::ITEM * sizeof(cx<float>));
-            small_dispatch(a, ld, item.a, item.b, S, so);
+            for (int g = tid; g < item.b; g += batched::NT) s_off[g] = a.off[a.group_tx[item.a + g]];
+            __syncthreads();
+            small_dispatch(a, ld.lgN, ld.tau, item.b, s_off, smem_raw);
             continue;
         }
-        const int key = item.len * 4 + item.kind;
-        if (tid == 0 && s_key != key) {
-            s_sa = (item.kind == 1) ? ld.s1 : ld.s2;
-            s_sa.in = (item.kind == 1) ? a.in : a.out;
-            s_sa.out = a.out;
-            s_sa.conj = a.conj;
-            s_key = key;
+        if (key != item.len * 4 + item.kind) {    // (the same for every thread)
+            key = item.len * 4 + item.kind;
+            const unsigned *src = reinterpret_cast<const unsigned *>(item.kind == 1 ? &ld.s1 : &ld.s2);
+            unsigned *dst = reinterpret_cast<unsigned *>(&s_sa);
+            for (int i = tid; i < (int)(sizeof(s_sa) / 4); i += batched::NT) dst[i] = src[i];
+            __syncthreads();
+            if (tid == 0) {
+                s_sa.in = static_cast<const cx<float> *>(item.kind == 1 ? a.in : a.out);
+                s_sa.out = static_cast<cx<float> *>(a.out);
+                s_sa.conj = a.conj;
+            }
         }
-        const StageArgs &sa = s_sa;
-        const long long boff = item.off;
         if (item.kind == 2) {
             if (tid == 0) {
                 const unsigned need = (unsigned)ld.ntiles1 + a.wait_bias;
@@ -427,10 +213,10 @@ __global__ void __launch_bounds__(batched::NT, MINB) paco_batched_kernel(const _
             }
             __syncthreads();
             if (!s_ok) continue;                  // reported through the status word
-            stage_dispatch<MINB, true>(sa, ld.lg2, item.b, boff, smem_raw);
+            stage_item<false>(s_sa, ld.lg2, item.b, item.off, smem_raw);
         } else {
             __syncthreads();                      // s_sa written
-            stage_dispatch<MINB, false>(sa, ld.lg1, item.b, boff, smem_raw);
+            stage_item<true>(s_sa, ld.lg1, item.b, item.off, smem_raw);
             __syncthreads();                      // every store of the tile issued
             if (tid == 0) {
                 __threadfence();
@@ -469,15 +255,39 @@ struct BatchedState {
     int tuned = 0;
 };
 
-static const void *batched_fn(int minb)
-{
-    return minb >= 2 ? (const void *)paco_batched_kernel<2> : (const void *)paco_batched_kernel<1>;
-}
+static const void *batched_fn() { return (const void *)paco_batched_kernel; }
 
-static int stage_smem_bytes(int lgL, int lgW, int mode)
+// The tile of a stage of length 2^lgL (its factors and columns) and what it and
+// a group of transforms of 2^lgN need of shared memory.
+template <int LG>
+static int stage_tile_of(bool first, FoldKernel *k)
 {
-    const int A = 1 << ((lgL + 1) / 2), B = 1 << (lgL / 2), W = 1 << lgW;
-    return stage_smem_elems(A, B, 1, W, mode == 1 ? 1 : W) * 8;
+    using C1 = StageCfgB<LG, true>;
+    using C2 = StageCfgB<LG, false>;
+    static_assert(C1::NT == batched::NT && C2::NT == batched::NT, "item size");
+    k->lgA = C1::LGA;
+    k->lgB = C1::LGB;
+    k->lgW = C1::LGW;
+    return first ? C1::SMEM : C2::SMEM;
+}
+static int stage_tile(int lgL, bool first, FoldKernel *k)
+{
+    switch (lgL) {
+    case 6: return stage_tile_of<6>(first, k);
+    case 7: return stage_tile_of<7>(first, k);
+    case 8: return stage_tile_of<8>(first, k);
+    case 9: return stage_tile_of<9>(first, k);
+    default: return stage_tile_of<10>(first, k);
+    }
+}
+static int small_smem(int lgN)
+{
+    using namespace batched;
+    constexpr int bytes[10] = {WholeCfg<4, EPT, NT>::SMEM,  WholeCfg<5, EPT, NT>::SMEM,  WholeCfg<6, EPT, NT>::SMEM,
+                               WholeCfg<7, EPT, NT>::SMEM,  WholeCfg<8, EPT, NT>::SMEM,  WholeCfg<9, EPT, NT>::SMEM,
+                               WholeCfg<10, EPT, NT>::SMEM, WholeCfg<11, EPT, NT>::SMEM, WholeCfg<12, EPT, NT>::SMEM,
+                               WholeCfg<13, EPT, NT>::SMEM};
+    return bytes[lgN - 4];
 }
 
 void batched_destroy(BatchedState *bs)
@@ -593,30 +403,30 @@ static void schedule_items(const std::vector<int64_t> &lengths, const std::vecto
 static paco_status_t build_device(paco_plan *pl, BatchedState *bs)
 {
     free_device(bs);
-    int nsm = pl->num_sms;
-    const void *fn = batched_fn(bs->minb);
-    // shared memory: the largest stage tile or a small group
-    int smem = batched::ITEM * 8 + (batched::ITEM / 16) * 8 + (128 + 64) * 8;
+    const void *fn = batched_fn();
+    // shared memory: the largest tile of the batch
+    int smem = 0;
+    FoldKernel k1, k2;
     for (int lg : bs->lgs) {
         const LenCfg &c = bs->cfg[lg];
-        if (lg <= batched::SMALL_MAX_LG) continue;
-        smem = std::max(smem, stage_smem_bytes(c.lg1, 13 - c.lg1, 1));
-        smem = std::max(smem, stage_smem_bytes(c.lg2, 13 - c.lg2, 2));
+        if (lg <= batched::SMALL_MAX_LG) smem = std::max(smem, small_smem(lg));
+        else smem = std::max(smem, std::max(stage_tile(c.lg1, true, &k1), stage_tile(c.lg2, false, &k2)));
     }
     bs->smem = smem;
     // the attribute belongs to the kernel, not to the plan: set to what any
     // configuration needs, so that a second plan does not lower the first one's
     int most = smem;
+    for (int lg = 4; lg <= batched::SMALL_MAX_LG; ++lg) most = std::max(most, small_smem(lg));
     for (int lgL = batched::STAGE_MIN_LG; lgL <= batched::STAGE_MAX_LG; ++lgL)
-        most = std::max(most, std::max(stage_smem_bytes(lgL, 13 - lgL, 1), stage_smem_bytes(lgL, 13 - lgL, 2)));
+        most = std::max(most, std::max(stage_tile(lgL, true, &k1), stage_tile(lgL, false, &k2)));
     PACO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     int occ = 0;
     PACO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, batched::NT, smem));
     if (occ < 1) return fail(PACO_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
     if (occ > bs->minb) occ = bs->minb;
-    bs->grid = nsm * occ;
+    bs->grid = pl->num_sms * occ;
 
-    // length descriptors and twiddle tables (FP64-generated)
+    // length descriptors and tables of factors (FP64-generated)
     std::vector<BLen> lens;
     std::map<int, int> len_index;
     for (int lg : bs->lgs) {
@@ -624,53 +434,25 @@ static paco_status_t build_device(paco_plan *pl, BatchedState *bs)
         BLen L;
         memset(&L, 0, sizeof(L));
         L.lgN = lg; L.lg1 = c.lg1; L.lg2 = c.lg2; L.t = c.t;
-        const long long N = 1LL << lg, N1 = 1LL << c.lg1, N2 = 1LL << c.lg2;
         paco_status_t st;
+        void *tw = nullptr;
         if (lg <= batched::SMALL_MAX_LG) {
             L.small = 1;
             L.G = batched::ITEM >> lg;
-            void *tw = nullptr;
-            if ((st = gen_table(8, &tw, N, N, 1, 0)) != PACO_OK) return st;
+            if ((st = whole_table(lg, &tw)) != PACO_OK) return st;
             bs->tables.push_back(tw);
-            L.twN = tw;
+            L.tau = static_cast<const float2 *>(tw);
         } else {
-            void *t1 = nullptr, *t2 = nullptr, *lo = nullptr, *hi = nullptr;
-            const int lob = (lg + 1) / 2;
-            const long long nlo = 1LL << lob, nhi = N / nlo;
-            if ((st = gen_table(8, &t1, N1, N1, 1, 0)) != PACO_OK) return st;
-            bs->tables.push_back(t1);
-            if ((st = gen_table(8, &t2, N2, N2, 1, 0)) != PACO_OK) return st;
-            bs->tables.push_back(t2);
-            if ((st = gen_table(8, &lo, N, nlo, 1, 0)) != PACO_OK) return st;
-            bs->tables.push_back(lo);
-            if ((st = gen_table(8, &hi, N, nhi, nlo, 0)) != PACO_OK) return st;
-            bs->tables.push_back(hi);
+            const int f[2] = {c.lg1, c.lg2};
             for (int s = 0; s < 2; ++s) {
-                StageArgs &a = s ? L.s2 : L.s1;
-                memset(&a, 0, sizeof(a));
-                const int lgL = s ? c.lg2 : c.lg1;
-                const long long Cc = s ? N1 : N2;
-                int lgW = 13 - lgL;
-                if ((1LL << lgW) > Cc) lgW = s ? c.lg1 : c.lg2;
-                a.batch_stride = N;
-                a.C = (int)Cc;
-                a.out_ld = (int)N1;
-                a.lgW = lgW;
-                a.lgK = 0;
-                a.mode = s ? 2 : 1;
-                a.rev_bits = c.lg2;
-                a.rev_t = c.t;
-                a.twL = s ? t2 : t1;
-                a.twN_lo = lo;
-                a.twN_hi = hi;
-                a.twN_lo_bits = lob;
-                a.N_mask = (unsigned)(N - 1);
-                a.pad = s ? (1 << lgW) : 1;
-                if (s) L.ntiles2 = (int)(Cc >> lgW);
-                else L.ntiles1 = (int)(Cc >> lgW);
-                if ((1LL << lgL) * (1LL << lgW) != batched::ITEM)
-                    return fail(PACO_ERR_UNSUPPORTED, "length 2^%d: stage tile is not %d elements", lg,
-                                batched::ITEM);
+                FoldKernel k;
+                stage_tile(f[s], s == 0, &k);
+                FoldArgs<float> &a = s ? L.s2 : L.s1;
+                fold_pass_args(&a, k, f, 2, s, c.t);
+                if ((st = fold_table<float>(&tw, k, s, s ? c.lg1 : 0)) != PACO_OK) return st;
+                bs->tables.push_back(tw);
+                a.tau = static_cast<const cx<float> *>(tw);
+                (s ? L.ntiles2 : L.ntiles1) = 1 << a.lg_all;
             }
         }
         len_index[lg] = (int)lens.size();
@@ -714,7 +496,7 @@ static paco_status_t launch(const paco_plan *pl, const BatchedState *bs, const v
     PACO_CUDA_TRY(cudaMemsetAsync(bs->d_ctr, 0, bs->ctr_words * sizeof(unsigned), stream));
     const int grid = std::min<long long>(bs->grid, std::max(1, bs->nitems));
     void *params[] = {&a};
-    PACO_CUDA_TRY(cudaLaunchKernel(batched_fn(bs->minb), dim3((unsigned)grid), dim3(batched::NT), params,
+    PACO_CUDA_TRY(cudaLaunchKernel(batched_fn(), dim3((unsigned)grid), dim3(batched::NT), params,
                                    (size_t)bs->smem, stream));
     return PACO_OK;
 }
@@ -737,9 +519,9 @@ void batched_info(const paco_plan *pl, paco_plan_info_t *info)
 
 // ---- autotuner ----------------------------------------------------------------
 // Times candidate configurations with CUDA events on plan-owned scratch
-// buffers and keeps the fastest: per length class (b and the N1 x N2 split,
-// on a sub-batch of that class alone), then the CTAs per SM and the Phase III
-// lag on a sub-batch of the whole mix.
+// buffers and keeps the fastest: per length class (the N1 x N2 split, on a
+// sub-batch of that class alone), then the CTAs per SM and the Phase III lag on
+// a sub-batch of the whole mix.
 static float time_config(paco_plan *pl, BatchedState *bs, const void *in, void *out, int reps)
 {
     if (build_device(pl, bs) != PACO_OK) return -1.f;
@@ -835,15 +617,14 @@ static paco_status_t autotune(paco_plan *pl, BatchedState *bs)
             if (upload_offsets(&sub) != PACO_OK) { result = PACO_ERR_CUDA; break; }
             float best = -1.f;
             LenCfg bestc = bs->cfg[lg];
-            for (int lg1 = 1; lg1 < lg; ++lg1) {
-                for (int t = 1; t <= 4; ++t) {
-                    LenCfg c;
-                    c.lg1 = lg1; c.lg2 = lg - lg1; c.t = t;
-                    if (!len_cfg_ok(lg, c)) continue;
-                    sub.cfg[lg] = c;
-                    const float ms = time_config(pl, &sub, in, out, 3);
-                    if (ms > 0.f && (best < 0.f || ms < best)) { best = ms; bestc = c; }
-                }
+            for (int lg1 = 1; lg1 < lg && lg > batched::SMALL_MAX_LG; ++lg1) {
+                LenCfg c;
+                c.lg1 = lg1; c.lg2 = lg - lg1; c.t = 4;
+                while (c.t > 1 && !len_cfg_ok(lg, c)) --c.t;
+                if (!len_cfg_ok(lg, c)) continue;
+                sub.cfg[lg] = c;
+                const float ms = time_config(pl, &sub, in, out, 3);
+                if (ms > 0.f && (best < 0.f || ms < best)) { best = ms; bestc = c; }
             }
             best_cfg[minb][lg] = bestc;
             free_device(&sub);

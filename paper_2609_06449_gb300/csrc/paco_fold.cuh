@@ -38,6 +38,7 @@
 // and takes the plain DFT (ROWS).
 #pragma once
 
+#include "../../include/paco.h"
 #include "paco_common.cuh"
 
 namespace paco {
@@ -182,14 +183,15 @@ __device__ __forceinline__ void fold_dft(cx<R> *v, const Tau &tau)
     for (int i = 0; i < RADIX; ++i) v[i] = u[i];
 }
 
-template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_>
+// EPT_: points a thread holds (0: 16, or 32 where a factor needs them).
+template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0>
 struct FoldCfg {
     using R = R_;
     static constexpr int LGA = LGA_, LGB = LGB_, LGW = LGW_;
     static constexpr bool FIRST = FIRST_;
     static constexpr int TW = FIRST_ ? 0 : TW_;
     static constexpr int A = 1 << LGA, B = 1 << LGB, W = 1 << LGW, L = A * B;
-    static constexpr int EPT = A > B ? (A > 16 ? A : 16) : (B > 16 ? B : 16);
+    static constexpr int EPT = EPT_ ? EPT_ : A > B ? (A > 16 ? A : 16) : (B > 16 ? B : 16);
     static constexpr int NT = L * W / EPT;
     static constexpr int U1 = EPT / A, U2 = EPT / B;
     // exchange layouts as in paco_pass.cuh; PH points make one shared-memory phase
@@ -399,6 +401,15 @@ FoldKernel fold_kernel_of()
     k.smem = CFG::SMEM;
     return k;
 }
+
+// The launch constants of pass i of the n factors f (log2; first pass first),
+// tables aside: k.lgA, k.lgB and k.lgW are read.
+template <typename R>
+void fold_pass_args(FoldArgs<R> *a, const FoldKernel &k, const int *f, int n, int i, int t);
+
+// A device table for FoldArgs::tau in mode FoldCfg::TW, 2^lgK columns.
+template <typename R>
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK);
 
 // The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
 // (the row stride); fn == nullptr where none is built.

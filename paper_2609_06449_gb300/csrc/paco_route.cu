@@ -92,7 +92,7 @@ static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, cudaStr
 
 // FoldArgs::tau in mode FoldCfg::TW over 2^lgK columns.
 template <typename R>
-static paco_status_t tau_table(void **dst, const FoldKernel &k, int mode, int lgK)
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK)
 {
     const int A = 1 << k.lgA, B = 1 << k.lgB, lgL = k.lgA + k.lgB;
     const bool fp64 = sizeof(R) == 8;
@@ -116,6 +116,8 @@ static paco_status_t tau_table(void **dst, const FoldKernel &k, int mode, int lg
     return PACO_OK;
 }
 
+template paco_status_t fold_table<float>(void **, const FoldKernel &, int, int);
+
 paco_status_t whole_table(int lgN, void **dst)
 {
     int k[4], n = 0, total = 0;                            // log2 of the frequencies known before every step
@@ -129,13 +131,11 @@ paco_status_t whole_table(int lgN, void **dst)
     return PACO_OK;
 }
 
-// Pass i of the n factors f (log2): its strides, row maps and tables.  Its
-// columns are the frequencies of the passes before it (the first pass: all
-// other rows of the view).
+// A pass's columns are the frequencies of the passes before it (the first
+// pass: all other rows of the view).
 template <typename R>
-static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, const int *f, int n, int i, int t)
+void fold_pass_args(FoldArgs<R> *a, const FoldKernel &k, const int *f, int n, int i, int t)
 {
-    const FoldKernel &k = r->k[i];
     memset(a, 0, sizeof(*a));
     int lgN = 0, lgK = 0;
     for (int j = 0; j < n; ++j) {
@@ -143,7 +143,7 @@ static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, c
         if (j < i) lgK += f[j];
     }
     const int lgL = f[i], lgC = i == 0 ? lgN - lgL : lgK;
-    a->bstride = pl->N;
+    a->bstride = 1LL << lgN;
     a->ld_in = 1u << lgC;
     a->ld_out = i == 0 ? 1u << lgL : 1u << lgC;
     a->rev_bits = i == 0 ? 0 : lgL;
@@ -155,12 +155,21 @@ static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, c
     a->lg_tiles = lgC - k.lgW;
     a->lg_all = lgN - lgL - k.lgW;
     a->blk_stride = i == 0 || i == n - 1 ? 0u : 1u << (lgK + lgL);
-    a->lo_bits = pl->twN_lo_bits;
     a->lg_n = lgN;
     a->lg_k = lgK;
     a->mult = R(1);
+}
+template void fold_pass_args<float>(FoldArgs<float> *, const FoldKernel &, const int *, int, int, int);
+
+// Pass i of the plan's route: launch constants and tables.
+template <typename R>
+static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, const int *f, int n, int i, int t)
+{
+    const FoldKernel &k = r->k[i];
+    fold_pass_args(a, k, f, n, i, t);
+    a->lo_bits = pl->twN_lo_bits;
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    paco_status_t st = tau_table<R>(&r->tw[i], k, r->twmode[i], lgK);
+    paco_status_t st = fold_table<R>(&r->tw[i], k, r->twmode[i], a->lg_k);
     a->tau = static_cast<const cx<R> *>(r->tw[i]);
     if (st != PACO_OK || r->twmode[i] != 2 || sizeof(R) == 8) return st;
     // w_N^{-r} in FP64, two levels

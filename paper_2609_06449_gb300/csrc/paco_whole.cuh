@@ -16,7 +16,6 @@
 // 8 + 8 -- 16 different banks (4-point rows aside).
 #pragma once
 
-#include "../../include/paco.h"
 #include "paco_fold.cuh"
 
 namespace paco {
