@@ -11,24 +11,28 @@
 //              input-slab-owner) and computes their length-256 DFTs in shared
 //              memory (radix 16 x 16);
 //   middle     each result A[v][c] takes the top-level twiddle w_N^{-vc} and
-//              goes straight to the CTA that owns output column v (its
-//              processor owns v by Eq. (3)), at row pi_m2(c) of that CTA's
-//              part of W = Z-hat (Eq. (17)): the fused digit reversal of
-//              PARA-CO-DRP (Sect. 4.2, App. C.5) as the addresses of one
-//              all-to-all through distributed shared memory -- N/K^2 items per
+//              goes to the CTA that owns output column v (its processor owns v
+//              by Eq. (3)): one all-to-all through distributed shared memory
+//              (PARA-CO-DRP, Sect. 4.2, App. C.5), one block of N/K^2 items per
 //              ordered pair of CTAs, N/p^2 per ordered pair of processors; a
-//              CTA's items for itself stay in its own shared memory;
+//              CTA's block for itself stays in its own shared memory.  Row
+//              pi_m2(c) of W = Z-hat (Eq. (17)) is kept as row c mod 256/K of
+//              the block from c's owner;
 //   Phase III  computes the length-256 DFTs of its output columns over the
-//              digit-reversed rows (Lemma 1, input layout) and writes columns
-//              k1 in [r 256/K, (r+1) 256/K) of Y = y viewed N2 x N1.
+//              digit-reversed rows pi_m2(j) (Lemma 1, input layout), that is
+//              over c = j, and writes columns k1 in [r 256/K, (r+1) 256/K) of
+//              Y = y viewed N2 x N1.
+// The blocks travel as one bulk copy each (2 KiB for K = 16), which counts its
+// bytes on the destination's transaction barrier.  Item by item (st.async of 8
+// bytes) the exchange kept each SM's port busy for 4096 packets a side: the
+// transform took 6.7 us in a replayed graph, and takes 6.05 us so.
 // Synchronisation: one split cluster barrier (arrive at entry, wait before the
-// first remote store) makes sure every CTA of the cluster runs and has set up
-// its transaction barrier; the all-to-all is asynchronous stores
-// (st.async) that count their bytes on the destination CTA's barrier, so a
-// CTA starts Phase III as soon as its own N/K items have landed, with no
-// second cluster-wide barrier.  The wait is bounded (2 s): a CTA that gives up
-// sets the plan's status word to PACO_ERR_TIMEOUT and finishes the launch with
-// whatever landed.
+// first copy) makes sure every CTA of the cluster runs and has set up its
+// barrier; a CTA starts Phase III as soon as its own N/K items have landed; a
+// second split barrier (arrive there, wait at the end) keeps each CTA's blocks
+// in place until all of them have been read.  The wait for the items is bounded
+// (2 s): a CTA that gives up sets the plan's status word to PACO_ERR_TIMEOUT and
+// finishes the launch with whatever landed.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -45,7 +49,6 @@ struct ClusterArgs {
     float2 *out;
     long long N;                 // 65536
     int p;                       // processors (counts are kept per pair of processors)
-    int rev_t;                   // digit reversal pi_m2 over 8 bits, t bits per digit
     int conj;                    // dir = +1: conjugate on load and store
     const float2 *tw256;         // w_256^{-r}, r < 256
     const float2 *twN;           // w_N^{-r}, r < N
@@ -81,12 +84,12 @@ __device__ __forceinline__ unsigned map_rank(unsigned addr, int rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// 8-byte store into another CTA's shared memory that counts its bytes on
-// that CTA's transaction barrier
-__device__ __forceinline__ void st_async_v2(unsigned addr, float x, float y, unsigned bar)
+// bulk copy into another CTA's shared memory that counts its bytes on that
+// CTA's transaction barrier
+__device__ __forceinline__ void bulk_copy(unsigned dst, unsigned src, unsigned bytes, unsigned bar)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-                 :: "r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity)
 {
@@ -102,27 +105,6 @@ __device__ __forceinline__ cx<float> cmul2(cx<float> a, float2 w)
 {
     return make_cx<float>(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
 }
-// Column swizzle of a row of a CTA's W part.  Row pi_m2(c) has the bits of
-// c's low nibble in its high nibble (for every digit width t | 4), so the 16
-// lanes of a half-warp, which hold 16 consecutive c, write 16 different
-// banks in the exchange, and read one row's 16 columns in Phase III.
-__device__ __forceinline__ int sw(int row) { return row >> 4; }
-
-// Rotate v left by r (0 <= r < 16, uniform across the warp) without dynamic
-// register indexing: out[k] = v[(k + r) & 15], four conditional shifts.
-__device__ __forceinline__ void rotate16(cx<float> *v, int r)
-{
-#pragma unroll
-    for (int b = 1; b < 16; b <<= 1) {
-        const bool on = (r & b) != 0;
-        cx<float> t[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) t[k] = on ? v[(k + b) & 15] : v[k];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = t[k];
-    }
-}
-
 // One length-256 DFT per column of a W-column block, as radix 16 x 16 with
 // one exchange through buf.  Pass 1: thread (col, t16) -- col = tid % W,
 // t16 = tid / W -- brings its 16 inputs x[t16 + 16 s] in v (the caller loads
@@ -158,7 +140,8 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
     extern __shared__ __align__(16) float2 smem[];
     constexpr int NK = 65536 / K;                             // items per CTA
     float2 *bufA = smem;                                      // the in-CTA exchanges of the length-256 DFTs
-    float2 *bufB = smem + NK;                                 // this CTA's part of W, filled by the all-to-all
+    float2 *bufB = smem + NK;                                 // this CTA's part of W, [source CTA][c][v], filled by the all-to-all
+    float2 *bufC = smem + 2 * NK;                             // what it sends, [destination CTA][c][v]
     __shared__ __align__(8) unsigned long long full;          // counts the bytes that land in bufB
     __shared__ unsigned cnt[16];
     constexpr int W1 = L / K, W2 = L / K;                     // input and output columns of a CTA
@@ -208,21 +191,21 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
     // v[k] = A[v][c] with c = cB, v = tB + 16 k (the natural frequency k1)
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = cmul2(v[k], wt[k]);  // Z[v][c] = A[v][c] w_N^{-vc}
-    const int row = (int)digit_reverse((unsigned)cB, 8, a.rev_t);   // pi_m2(c): its row of W
-    // Send order: warp w of CTA q starts at k = (q + w) mod 16, so that at
-    // every step the CTAs' stores spread over all destinations; the 16 lanes
-    // of a half-warp fill 16 consecutive columns of one destination row.
-    const int rho = ((int)q + (tid >> 5)) & 15;
-    rotate16(v, rho);
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // all CTAs run, barriers set up
-    const unsigned bufB_a = smem_u32(bufB);
+    // k-th result: column v = tB + 16 k of Y, row colB of the block for v's owner
+    // (16 lanes fill 16 consecutive places)
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const int vf = tB + 16 * ((j + rho) & 15);            // k1 = v
-        const int qd = vf / W2, vl = vf % W2;                 // the CTA that owns output column v, local column
-        const unsigned dst = map_rank(bufB_a + (unsigned)(row * W2 + (vl ^ sw(row))) * 8u, qd);
-        st_async_v2(dst, v[j].x, v[j].y, map_rank(fullA, qd));
+    for (int k = 0; k < 16; ++k) {
+        const int vf = tB + 16 * k, qd = vf / W2, vl = vf % W2;
+        bufC[(qd * W1 + colB) * W2 + vl] = make_float2(v[k].x, v[k].y);
         if (a.pair_count) atomicAdd(&cnt[qd], 1u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // the copies below read these stores
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // all CTAs run, barriers set up
+    __syncthreads();
+    if (tid < K) {
+        const int qd = ((int)q + tid) % K;                    // spread over the destinations
+        constexpr unsigned block = W1 * W2 * sizeof(float2);
+        bulk_copy(map_rank(smem_u32(bufB) + q * block, qd), smem_u32(bufC) + qd * block, block, map_rank(fullA, qd));
     }
     // every item of this CTA's part has landed (bounded wait)
     if (!mbar_try_wait(fullA, 0)) {
@@ -234,6 +217,9 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
             }
         }
     }
+    __syncwarp();
+    // this CTA has what the others sent it (or gave up waiting)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     if (a.pair_count) {                                       // per ordered pair of processors
         __syncthreads();
         if (tid < K) {
@@ -242,12 +228,12 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
         }
     }
 
-    // ---- Phase III on output columns v = q W2 + vl, logical rows j -> pi_m2(j)
+    // ---- Phase III on output columns v = q W2 + vl, logical rows j = c
     const int vl = col, u16 = t16;
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
-        const int rj = (int)digit_reverse((unsigned)(u16 + 16 * s), 8, a.rev_t);
-        v[s] = ld_cx(&bufB[rj * W2 + (vl ^ sw(rj))]);
+        const int j = u16 + 16 * s;
+        v[s] = ld_cx(&bufB[j * W2 + vl]);                     // row j mod W1 of the block from CTA j / W1
     }
     dft256_cols<false>(v, bufA, W2, vl, u16, tw);
     const int k1 = (int)q * W2 + vl;
@@ -256,6 +242,7 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
         const int k2 = u16 + 16 * k;
         y[(long long)k2 * L + k1] = make_float2(v[k].x, a.conj ? -v[k].y : v[k].y);   // Y[k2][k1] = y[k1 + k2 N1]
     }
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");   // every block of this CTA has been read
 }
 
 const void *cluster_kernel_fn(int K)
@@ -292,7 +279,7 @@ int cluster_size()
         memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3(16, 1, 1);
         cfg.blockDim = dim3(256, 1, 1);
-        cfg.dynamicSmemBytes = 2 * 4096 * sizeof(float2);
+        cfg.dynamicSmemBytes = 3 * 4096 * sizeof(float2);
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 16;
@@ -317,7 +304,6 @@ paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int
     a.out = static_cast<float2 *>(out);
     a.N = pl->N;
     a.p = pl->p;
-    a.rev_t = pl->t;
     a.conj = (dir == 1);
     a.tw256 = static_cast<const float2 *>(pl->twL2);
     a.twN = static_cast<const float2 *>(pl->twN_full);
@@ -327,7 +313,7 @@ paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int
     a.extra_tx = 8u * pl->dbg_wait_bias;          // paco_debug_set_waits: a wait that runs out
     const int K = pl->fused_k;                    // chosen at plan creation on the plan's device
     const int threads = (int)(pl->N / K / 16);
-    const size_t smem = 2 * (size_t)(pl->N / K) * sizeof(float2);
+    const size_t smem = 3 * (size_t)(pl->N / K) * sizeof(float2);
     for (int64_t b0 = 0; b0 < pl->batch; b0 += 8192) {
         const int64_t nb = (pl->batch - b0 < 8192) ? pl->batch - b0 : 8192;
         ClusterArgs ab = a;
@@ -358,9 +344,9 @@ paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int
 paco_status_t cluster_setup(paco_plan *pl)
 {
     PACO_CUDA_TRY(cudaFuncSetAttribute(cluster_kernel_fn(8), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       2 * 8192 * (int)sizeof(float2)));
+                                       3 * 8192 * (int)sizeof(float2)));
     PACO_CUDA_TRY(cudaFuncSetAttribute(cluster_kernel_fn(16), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       2 * 4096 * (int)sizeof(float2)));
+                                       3 * 4096 * (int)sizeof(float2)));
     pl->fused_k = cluster_size();
     return gen_table(8, &pl->twN_full, (pl->dims >= 2) ? 1 : pl->N, pl->N, 1, 0);   // ones for the 2-D DFT
 }

@@ -62,6 +62,7 @@ struct FoldArgs {
     int lo_bits;
     int lg_n, lg_k;         // log2 N, log2 K
     int conj;               // 1: the conjugate transform
+    int reverse;            // 1: tiles from the last to the first
     R mult;                 // FIRST: the input is scaled by mult * (*scale or 1)
     const double *scale;
 };
@@ -212,8 +213,15 @@ struct FoldCfg {
     static constexpr int MINB = REGS_CTAS < 1 ? 1 : (REGS_CTAS < SMEM_CTAS ? REGS_CTAS : SMEM_CTAS);
 };
 
-// One tile of the transform at element offset boff.
-template <class CFG>
+// Programmatic dependent launch: the next kernel of the stream may start its
+// CTAs (they read tables only) as this one's last ones run; grid_wait holds
+// until the kernels before are complete.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// One tile of the transform at element offset boff (PDL: the tile's kernel was
+// launched with programmatic serialisation).
+template <class CFG, bool PDL = false>
 __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, int tile, long long boff,
                                           unsigned char *smem_raw)
 {
@@ -261,6 +269,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
     };
     if constexpr (TW == 2 && CFG::EPT == 32) load_twiddles();
 
+    if constexpr (PDL) grid_wait();
     // ---- F1
     C v[CFG::EPT];
 #pragma unroll
@@ -371,7 +380,8 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             V o;
             o.x = a.conj ? y.y : y.x;
             o.y = a.conj ? y.x : y.y;
-            q[FIRST ? (unsigned)(A * k) : a.rowK[k]] = o;
+            if constexpr (FIRST) q[A * k] = o;
+            else __stcs(q + a.rowK[k], o);
         }
     }
 }
@@ -380,7 +390,11 @@ template <class CFG>
 __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __grid_constant__ FoldArgs<typename CFG::R> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fold_tile<CFG>(a, (int)(blockIdx.x & ((1u << a.lg_all) - 1u)), (long long)(blockIdx.x >> a.lg_all) * a.bstride, smem_raw);
+    // every second pass takes the tiles from the end: what the pass before it
+    // wrote last is still in L2
+    grid_launch_dependents();
+    const unsigned b = a.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+    fold_tile<CFG, true>(a, (int)(b & ((1u << a.lg_all) - 1u)), (long long)(b >> a.lg_all) * a.bstride, smem_raw);
 }
 
 // What the host needs to launch one of the kernels above.
@@ -413,7 +427,7 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK);
 
 // The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
 // (the row stride); fn == nullptr where none is built.
-FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC);
+FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC, bool narrow);
 FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC);
 
 } // namespace paco

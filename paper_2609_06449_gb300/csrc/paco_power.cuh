@@ -14,7 +14,7 @@
 // instructions a point on run-time strides and twiddle products.
 #pragma once
 
-#include "paco_common.cuh"
+#include "paco_fold.cuh"
 
 namespace paco {
 
@@ -34,6 +34,7 @@ struct PowerArgs {
     int lo_bits;
     unsigned n_mask;        // N - 1
     int conj;               // 1: the conjugate transform
+    int reverse;            // 1: tiles from the last to the first (what the pass before wrote last is in L2)
     const float *w;         // Phase III: *loss += sum over n of w[n] |out[n]|^2, and
     double *loss;
     int store_weighted;     //   (1) w[n] * out[n] is stored in place of out[n]
@@ -178,11 +179,14 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_power_kernel(const __
     C *sm = reinterpret_cast<C *>(smem_raw);
     C *tab = sm + CFG::EX;
     const int tid = threadIdx.x;
-    const long long boff = (long long)(blockIdx.x >> a.lg_all) * a.bstride;
-    const unsigned c0 = (blockIdx.x & ((1u << a.lg_all) - 1u)) << CFG::LGW;
+    grid_launch_dependents();
+    const unsigned bid = a.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+    const long long boff = (long long)(bid >> a.lg_all) * a.bstride;
+    const unsigned c0 = (bid & ((1u << a.lg_all) - 1u)) << CFG::LGW;
     const long long base = boff + c0;
     const float sg = a.conj ? -1.f : 1.f;
 
+    grid_wait();
     // ---- F1
     C v[EPT];
 #pragma unroll

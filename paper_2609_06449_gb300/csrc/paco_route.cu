@@ -19,6 +19,7 @@
 #include "paco_power.cuh"
 #include "paco_plan.h"
 #include "paco_stage_args.cuh"
+#include "paco_tcpass.cuh"
 #include "paco_whole.cuh"
 
 namespace paco {
@@ -33,6 +34,7 @@ struct Route {
     int twmode[MAX_PASSES] = {};       // FoldCfg::TW
     FoldArgs<float> f[MAX_PASSES];     // by the plan's precision
     FoldArgs<double> d[MAX_PASSES];
+    TcPassArgs t[MAX_PASSES];
     PowerKernel pk[2];              // the stages of the weighted power (fn == nullptr: the stage kernels)
     PowerArgs pa[2];
     void *tw[MAX_PASSES + 2] = {};     // the factors of every pass, w_L^{-r} of the two stages
@@ -228,18 +230,53 @@ static int route_factors(const paco_plan *pl, int lg1, int lg2, int *f)
     return n;
 }
 
+// The passes of a tensor-core form: 2^5..2^8 points each, at most four
+// contractions in all (the stage kernels' number: the error is theirs).
+static paco_status_t tc_setup(paco_plan *pl, Route *r, int lgN)
+{
+    int f[MAX_PASSES], n = (lgN + 7) / 8;
+    for (int i = 0, left = lgN; i < n; ++i) {
+        f[i] = (left + n - i - 1) / (n - i);
+        left -= f[i];
+    }
+    int t = pl->t, extra = 4 - n;
+    for (int i = 1; i < n; ++i)
+        if (f[i] % t) t = 1;
+    for (int i = 0, lgK = 0; i < n; lgK += f[i], ++i) {
+        const bool tc2 = f[i] == 8 && extra-- > 0;
+        r->k[i] = tcpass_kernel(pl->form, i == 0, tc2, f[i], i == 0 ? lgN - f[0] : lgK);
+        if (!r->k[i].fn) return PACO_OK;
+        TcPassArgs &a = r->t[i];
+        fold_pass_args(&a.f, r->k[i], f, n, i, t);
+        a.f.lo_bits = pl->twN_lo_bits;
+        a.lo = static_cast<const cx<float> *>(pl->twN_lo);
+        a.hi = static_cast<const cx<float> *>(pl->twN_hi);
+        a.frag = static_cast<const uint4 *>(pl->tc);
+        PACO_CUDA_TRY(cudaFuncSetAttribute(r->k[i].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->k[i].smem));
+        const paco_status_t st = gen_table(8, &r->tw[i], 1LL << f[i], 1LL << f[i], 1, 0);
+        if (st != PACO_OK) return st;
+        a.twL = static_cast<const cx<float> *>(r->tw[i]);
+    }
+    r->n = n;
+    return PACO_OK;
+}
+
 // Builds pl->route; its n stays 0 where the stage kernels run the plan.
 paco_status_t route_setup(paco_plan *pl)
 {
     // the plain forms with no stage option asked for
-    if (pl->form || pl->shard_G || pl->req_split || pl->req_ctas || pl->req_tile) return PACO_OK;
+    if (pl->shard_G || pl->req_split || pl->req_ctas || pl->req_tile) return PACO_OK;
     Route *r = new (std::nothrow) Route();
     if (!r) return fail(PACO_ERR_NOMEM, "out of host memory");
     pl->route = r;                                     // freed with the plan
     const int lg[2] = {ilog2_exact(pl->N1), ilog2_exact(pl->N2)}, lgN = lg[0] + lg[1];
+    if (pl->form) return pl->dims == 1 ? tc_setup(pl, r, lgN) : PACO_OK;
     int f[MAX_PASSES] = {0, 0, 0, 0};
-    // short transforms: one CTA holds them whole
-    if (pl->dims == 1 && pl->esize == 8 && (r->whole = whole_kernel(lgN)).fn) {
+    // short transforms: one CTA holds them whole (a few of 2^13 or 2^14 points
+    // spread better over the SMs in two passes: one 2^14 7.9 and 4.9 us, 40 of
+    // them 8.5 and 8.4, 100 8.6 and 10.9)
+    const bool whole = pl->dims == 1 && pl->esize == 8 && (lgN < 13 || pl->batch >= 32);
+    if (whole && (r->whole = whole_kernel(lgN)).fn) {
         const paco_status_t st = whole_table(lgN, &r->tw[0]);
         if (st != PACO_OK) return st;
         PACO_CUDA_TRY(cudaFuncSetAttribute(r->whole.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->whole.smem));
@@ -249,7 +286,7 @@ paco_status_t route_setup(paco_plan *pl)
     for (int i = 0, lgK = 0; i < n; lgK += f[i], ++i) {
         const int lgC = i == 0 ? lgN - f[0] : lgK;
         r->twmode[i] = i == 0 || pl->dims >= 2 ? 0 : lgK + f[i] <= DIRECT_LG ? 1 : 2;
-        r->k[i] = pl->esize == 8 ? fold_kernel_f32(i == 0, r->twmode[i], f[i], lgC)
+        r->k[i] = pl->esize == 8 ? fold_kernel_f32(i == 0, r->twmode[i], f[i], lgC, pl->N * pl->batch <= (int64_t)1 << 24)
                                  : fold_kernel_f64(i == 0, r->twmode[i], f[i], lgC);
         if (!r->k[i].fn) n = 0;
     }
@@ -271,13 +308,26 @@ paco_status_t route_setup(paco_plan *pl)
 
 int route_passes(const paco_plan *pl) { return pl->route ? pl->route->n : 0; }
 
-static paco_status_t launch(const paco_plan *pl, const void *fn, void *args, int lg_all, int threads, int smem,
-                            cudaStream_t stream)
+static paco_status_t launch(const paco_plan *pl, const void *fn, void *args, long long ctas, int threads, int smem,
+                            bool pdl, cudaStream_t stream)
 {
-    const long long tiles = (long long)pl->batch << lg_all;
-    if (tiles > INT32_MAX) return fail(PACO_ERR_UNSUPPORTED, "batch of %lld transforms is too large", (long long)pl->batch);
+    if (ctas > INT32_MAX) return fail(PACO_ERR_UNSUPPORTED, "batch of %lld transforms is too large", (long long)pl->batch);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = stream;
+    // Programmatic serialisation from two CTAs an SM on (77 x 2^18: 111 -> 106
+    // us): a smaller grid's CTAs would be placed beside the ones still running
+    // instead of one to an SM (2^20: 12.3 -> 14.6 us).
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol)
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl && ctas > 2 * pl->num_sms ? 1 : 0;
     void *params[] = {args};
-    PACO_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)tiles), dim3((unsigned)threads), params, (size_t)smem, stream));
+    PACO_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, params));
     return PACO_OK;
 }
 
@@ -291,11 +341,12 @@ static paco_status_t run_passes(const paco_plan *pl, const FoldArgs<R> *args, co
         a.in = static_cast<const cx<R> *>(i == 0 ? in : out);
         a.out = static_cast<cx<R> *>(out);
         a.conj = dir == 1;
+        a.reverse = i & 1;
         if (terms && i == 0) {
             a.mult = (R)terms->ld_mult;
             a.scale = terms->ld_scale;
         }
-        const paco_status_t st = launch(pl, r.k[i].fn, &a, a.lg_all, r.k[i].threads, r.k[i].smem, stream);
+        const paco_status_t st = launch(pl, r.k[i].fn, &a, (long long)pl->batch << a.lg_all, r.k[i].threads, r.k[i].smem, true, stream);
         if (st != PACO_OK) return st;
     }
     return PACO_OK;
@@ -314,10 +365,20 @@ paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir,
         a.conj = dir == 1;
         a.mult = terms ? terms->ld_mult : 1.f;
         a.scale = terms ? terms->ld_scale : nullptr;
-        void *params[] = {&a};
-        const long long ctas = (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta;
-        PACO_CUDA_TRY(cudaLaunchKernel(r.whole.fn, dim3((unsigned)ctas), dim3((unsigned)r.whole.threads), params,
-                                       (size_t)r.whole.smem, stream));
+        return launch(pl, r.whole.fn, &a, (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta, r.whole.threads,
+                      r.whole.smem, true, stream);
+    }
+    if (pl->form) {
+        for (int i = 0; i < r.n; ++i) {
+            TcPassArgs a = r.t[i];
+            a.f.in = static_cast<const cx<float> *>(i == 0 ? in : out);
+            a.f.out = static_cast<cx<float> *>(out);
+            a.f.conj = dir == 1;
+            a.f.reverse = i & 1;
+            const paco_status_t st = launch(pl, r.k[i].fn, &a, (long long)pl->batch << a.f.lg_all, r.k[i].threads,
+                                            r.k[i].smem, true, stream);
+            if (st != PACO_OK) return st;
+        }
         return PACO_OK;
     }
     return pl->esize == 8 ? run_passes(pl, pl->route->f, in, out, dir, terms, stream)
@@ -337,7 +398,8 @@ paco_status_t route_power(const paco_plan *pl, int stage, const void *in, void *
     a.w = terms.st_w;
     a.loss = terms.st_loss;
     a.store_weighted = terms.st_weighted;
-    return launch(pl, k.fn, &a, a.lg_all, k.threads, k.smem, stream);
+    a.reverse = stage;
+    return launch(pl, k.fn, &a, (long long)pl->batch << a.lg_all, k.threads, k.smem, true, stream);
 }
 
 } // namespace paco

@@ -64,6 +64,21 @@ def test_double_passes_against_oracle(l1, l2, b, batch, passes, d):
 
 
 @pytest.mark.parametrize("d", [-1, 1])
+@pytest.mark.parametrize("form,tol", [(paco.C64_TC_BF16X3, None), (paco.C64_TC_FP16, 1e-3)])
+@pytest.mark.parametrize("l1,l2,b,batch", [(8, 8, 16, 3), (8, 9, 2, 2), (9, 9, 8, 1), (10, 9, 2, 1), (10, 10, 2, 3),
+                                           (11, 10, 2, 1), (11, 11, 2, 1), (12, 11, 2, 1), (12, 12, 4, 1), (13, 12, 2, 1)])
+def test_tensor_core_passes(l1, l2, b, batch, form, tol, d):
+    """Every length and place of a tensor-core pass (16 x 2, 4, 8, 16; first,
+    middle, last; F2 contracted and plain), the forms' own bounds."""
+    N = 1 << (l1 + l2)
+    plan = paco.Plan(1 << l1, 1 << l2, b, batch, form)
+    assert plan.info.passes == (l1 + l2 + 7) // 8
+    x = gaussian(batch * N, l1 + 31 * l2, np.complex64).reshape(batch, N)
+    ref = oracle.fft(x.astype(np.complex128), dir=d, threads=0)
+    assert _err(_run(plan, x, d), ref) <= (tol or 5e-7 * math.log2(N))
+
+
+@pytest.mark.parametrize("d", [-1, 1])
 @pytest.mark.parametrize("l1,l2,b", [(5, 6, 2), (6, 5, 2), (7, 8, 2), (8, 4, 4), (10, 9, 2), (9, 10, 2)])
 def test_passes_2d(l1, l2, b, d):
     batch, N1, N2 = 3, 1 << l1, 1 << l2

@@ -160,3 +160,38 @@ def test_whole_transform_exchanges(lg):
     ref = np.fft.fft(x, axis=1)
     assert np.max(np.abs(out - ref)) <= 1e-13 * np.max(np.abs(ref))
     assert conflicts <= (1 if lg >= 6 and lg != 9 else 2)
+
+
+@pytest.mark.parametrize("K", [8, 16])
+def test_cluster_block_exchange(K):
+    """paco_cluster.cu: CTA q's results in [destination][c][v] blocks, one copy a
+    pair of CTAs into [source][c][v], Phase III over rows j = c -- every place
+    written once, runs of 16 places a half-warp, and the DFT as the result."""
+    L, W = 256, 256 // K
+    rng = np.random.default_rng(2)
+    x = rng.normal(size=L * L) + 1j * rng.normal(size=L * L)
+    X = x.reshape(L, L)
+    tid = np.arange(4096 // K)
+    send = np.full((K, K * W * W), np.nan, complex)
+    for q in range(K):
+        col_b, t_b = tid // 16, tid % 16
+        A = np.fft.fft(X[:, q * W + col_b], axis=0)               # [v][thread]
+        for k in range(16):
+            v = t_b + 16 * k
+            place = ((v // W) * W + col_b) * W + v % W
+            assert all(len(set(place[h:h + 16] % 16)) == 16 for h in range(0, len(tid), 16))
+            assert np.all(np.isnan(send[q, place].real))
+            send[q, place] = A[v, tid] * np.exp(-2j * np.pi * v * (q * W + col_b) / L ** 2)
+    assert not np.any(np.isnan(send.real))
+    recv = send.reshape(K, K, W * W).transpose(1, 0, 2).reshape(K, K * W * W)
+    y = np.empty((L, L), complex)                                 # [k2][k1]
+    for q in range(K):
+        vl, u = tid % W, tid // W
+        cols = np.empty((L, W), complex)
+        for s in range(16):
+            place = (u + 16 * s) * W + vl
+            assert all(len(set(place[h:h + 16] % 16)) == 16 for h in range(0, len(tid), 16))
+            cols[u + 16 * s, vl] = recv[q, place]
+        y[:, q * W:(q + 1) * W] = np.fft.fft(cols, axis=0)
+    ref = np.fft.fft(x)
+    assert np.max(np.abs(y.reshape(-1) - ref)) <= 1e-12 * np.max(np.abs(ref))
