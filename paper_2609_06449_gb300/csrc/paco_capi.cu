@@ -463,7 +463,7 @@ extern "C" void paco_plan_destroy(paco_plan_t *pl)
     cudaFree(pl->twL2);
     cudaFree(pl->twN_lo);
     cudaFree(pl->twN_hi);
-    cudaFree(pl->twN_full);
+    cudaFree(pl->cluster_tau);
     cudaFree(pl->tw_ones);
     cudaFree(pl->split_scratch);
     for (int k = 0; k < 2; ++k)

@@ -10,9 +10,8 @@
 //              N1 x N2 (processor q = floor(r p / K) owns slab q, Eq.
 //              input-slab-owner) and computes their length-256 DFTs in shared
 //              memory (radix 16 x 16);
-//   middle     each result A[v][c] takes the top-level twiddle w_N^{-vc} and
-//              goes to the CTA that owns output column v (its processor owns v
-//              by Eq. (3)): one all-to-all through distributed shared memory
+//   middle     each result A[v][c] goes to the CTA that owns output column v (its
+//              processor owns v by Eq. (3)): one all-to-all through distributed shared memory
 //              (PARA-CO-DRP, Sect. 4.2, App. C.5), one block of N/K^2 items per
 //              ordered pair of CTAs, N/p^2 per ordered pair of processors; a
 //              CTA's block for itself stays in its own shared memory.  Row
@@ -20,7 +19,8 @@
 //              the block from c's owner;
 //   Phase III  computes the length-256 DFTs of its output columns over the
 //              digit-reversed rows pi_m2(j) (Lemma 1, input layout), that is
-//              over c = j, and writes columns k1 in [r 256/K, (r+1) 256/K) of
+//              over c = j, with the top-level twiddle w_N^{-vc} folded into their
+//              butterflies (paco_fold.cuh), and writes columns k1 in [r 256/K, (r+1) 256/K) of
 //              Y = y viewed N2 x N1.
 // The blocks travel as one bulk copy each (2 KiB for K = 16), which counts its
 // bytes on the destination's transaction barrier.  Item by item (st.async of 8
@@ -39,7 +39,7 @@
 #include <cstring>
 
 #include "../../include/paco.h"
-#include "paco_common.cuh"
+#include "paco_fold.cuh"
 #include "paco_plan.h"
 
 namespace paco {
@@ -50,8 +50,7 @@ struct ClusterArgs {
     long long N;                 // 65536
     int p;                       // processors (counts are kept per pair of processors)
     int conj;                    // dir = +1: conjugate on load and store
-    const float2 *tw256;         // w_256^{-r}, r < 256
-    const float2 *twN;           // w_N^{-r}, r < N
+    const float2 *tau;           // the factors of paco_fold.cuh: Phase I's F2 (128), Phase III's F1 and F2 (136 x 256)
     int *status;                 // device status word (PACO_ERR_TIMEOUT)
     unsigned *pair_count;        // p x p counts of items sent (test hook), or nullptr
     unsigned long long wait_ns;  // limit of the bounded wait
@@ -101,26 +100,17 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity)
     return ok != 0;
 }
 
-__device__ __forceinline__ cx<float> cmul2(cx<float> a, float2 w)
-{
-    return make_cx<float>(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
-}
 // One length-256 DFT per column of a W-column block, as radix 16 x 16 with
 // one exchange through buf.  Pass 1: thread (col, t16) -- col = tid % W,
-// t16 = tid / W -- brings its 16 inputs x[t16 + 16 s] in v (the caller loads
-// them) and the 15 inner twiddles w_256^{-s t16}, s = 1..15, in tw.  Pass 2:
+// t16 = tid / W -- brings the DFT of its 16 inputs x[t16 + 16 s] in v.  Pass 2:
 // thread (col2, u) -- (tid % W, tid / W) when T16_FAST is false, else
 // (tid / 16, tid % 16) -- gets outputs u + 16 k', k' < 16, of column col2 in
-// v.  buf holds the intermediate (k16, t16) of column col at row
-// 16 k16 + t16, column col ^ k16: conflict-free for both pass-2 roles.
+// v, with the factors f of its folded butterflies.  buf holds the intermediate
+// (k16, t16) of column col at row 16 k16 + t16, column col ^ k16:
+// conflict-free for both pass-2 roles.
 template <bool T16_FAST>
-__device__ __forceinline__ void dft256_cols(cx<float> *v, float2 *buf, int W, int col, int t16,
-                                            const float2 *tw)
+__device__ __forceinline__ void dft256_finish(cx<float> *v, float2 *buf, int W, int col, int t16, const float2 *f)
 {
-    dft16(v);
-#pragma unroll
-    for (int s = 1; s < 16; ++s) v[s] = cmul2(v[s], tw[s - 1]);
-    __syncthreads();                                          // the loads from buf are done
 #pragma unroll
     for (int s = 0; s < 16; ++s) buf[(s * 16 + t16) * W + (col ^ s)] = make_float2(v[s].x, v[s].y);
     __syncthreads();
@@ -128,7 +118,7 @@ __device__ __forceinline__ void dft256_cols(cx<float> *v, float2 *buf, int W, in
     const int col2 = T16_FAST ? tid / 16 : tid % W, u = T16_FAST ? tid % 16 : tid / W;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = ld_cx(&buf[(u * 16 + t) * W + (col2 ^ u)]);
-    dft16(v);
+    fold_dft<false, float, 16>(v, [&](int q) { return make_cx<float>(f[q].x, f[q].y); });
 }
 
 } // namespace
@@ -151,7 +141,7 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
     const int tid = threadIdx.x;
     const int col = tid % W1, t16 = tid / W1;                 // Phase I pass 1; Phase III: (vl, u16) = (col, t16)
     const int colB = tid / 16, tB = tid % 16;                 // Phase I pass 2: column q W1 + colB, outputs tB + 16 k
-    const int cglob = (int)q * W1 + col, cB = (int)q * W1 + colB;
+    const int cglob = (int)q * W1 + col;
     const unsigned fullA = smem_u32(&full);
 
     if (tid == 0) {
@@ -164,14 +154,16 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
     // (the barrier's initialisation is ordered by the fence above)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
-    // Twiddles first: the plan's tables are not written by the preceding
+    // Factors first: the plan's tables are not written by the preceding
     // kernels, so their loads overlap the wait for those kernels.
-    float2 tw[15];                                            // w_256^{-s t16}: the same in both phases
+    const int k1 = (int)q * W2 + col;                         // Phase III's column
+    float2 f1[8], f3a[8], f3b[8];
 #pragma unroll
-    for (int s = 1; s < 16; ++s) tw[s - 1] = __ldg(&a.tw256[(s * t16) & 255]);
-    float2 wt[16];                                            // w_N^{-vc}, v = tB + 16 k, c = cB (vc < N)
-#pragma unroll
-    for (int k = 0; k < 16; ++k) wt[k] = __ldg(&a.twN[(tB + 16 * k) * cB]);
+    for (int i = 0; i < 8; ++i) {
+        f1[i] = __ldg(&a.tau[i * 16 + tB]);
+        f3a[i] = __ldg(&a.tau[128 + i * L + k1]);
+        f3b[i] = __ldg(&a.tau[128 + (8 + i * 16 + t16) * L + k1]);
+    }
     // Programmatic dependent launch: wait for the kernels before this one
     // (they may write x or read y), then let the next kernel start its CTAs.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -187,10 +179,8 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
         v[s] = ld_cx(x + (long long)(t16 + 16 * s) * L + cglob);   // row t16 + 16 s of X
         if (a.conj) v[s].y = -v[s].y;
     }
-    dft256_cols<true>(v, bufA, W1, col, t16, tw);
-    // v[k] = A[v][c] with c = cB, v = tB + 16 k (the natural frequency k1)
-#pragma unroll
-    for (int k = 0; k < 16; ++k) v[k] = cmul2(v[k], wt[k]);  // Z[v][c] = A[v][c] w_N^{-vc}
+    dft16(v);
+    dft256_finish<true>(v, bufA, W1, col, t16, f1);
     // k-th result: column v = tB + 16 k of Y, row colB of the block for v's owner
     // (16 lanes fill 16 consecutive places)
 #pragma unroll
@@ -235,8 +225,8 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
         const int j = u16 + 16 * s;
         v[s] = ld_cx(&bufB[j * W2 + vl]);                     // row j mod W1 of the block from CTA j / W1
     }
-    dft256_cols<false>(v, bufA, W2, vl, u16, tw);
-    const int k1 = (int)q * W2 + vl;
+    fold_dft<false, float, 16>(v, [&](int i) { return make_cx<float>(f3a[i].x, f3a[i].y); });
+    dft256_finish<false>(v, bufA, W2, vl, u16, f3b);          // (every read of bufA was before the exchange)
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const int k2 = u16 + 16 * k;
@@ -305,8 +295,7 @@ paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int
     a.N = pl->N;
     a.p = pl->p;
     a.conj = (dir == 1);
-    a.tw256 = static_cast<const float2 *>(pl->twL2);
-    a.twN = static_cast<const float2 *>(pl->twN_full);
+    a.tau = static_cast<const float2 *>(pl->cluster_tau);
     a.status = pl->d_status;
     a.pair_count = pair_count;
     a.wait_ns = 2000000000ull;
@@ -340,7 +329,7 @@ paco_status_t launch_cluster(const paco_plan *pl, const void *in, void *out, int
     return PACO_OK;
 }
 
-// Kernel attributes and the plan's full table of w_N^{-r}, r < N (512 KiB).
+// Kernel attributes and the plan's table of factors (273 KiB).
 paco_status_t cluster_setup(paco_plan *pl)
 {
     PACO_CUDA_TRY(cudaFuncSetAttribute(cluster_kernel_fn(8), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -348,7 +337,20 @@ paco_status_t cluster_setup(paco_plan *pl)
     PACO_CUDA_TRY(cudaFuncSetAttribute(cluster_kernel_fn(16), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        3 * 4096 * (int)sizeof(float2)));
     pl->fused_k = cluster_size();
-    return gen_table(8, &pl->twN_full, (pl->dims >= 2) ? 1 : pl->N, pl->N, 1, 0);   // ones for the 2-D DFT
+    // the factors of two passes of 16 x 16 points, in one table
+    FoldKernel k;
+    k.lgA = k.lgB = 4;
+    void *t1 = nullptr, *t2 = nullptr;
+    paco_status_t st = fold_table<float>(&t1, k, 0, 0);
+    if (st == PACO_OK) st = fold_table<float>(&t2, k, 1, 8, pl->dims >= 2);   // (the 2-D DFT has no top-level twiddle)
+    cudaError_t e = cudaSuccess;
+    if (st == PACO_OK && (e = cudaMalloc(&pl->cluster_tau, (128 + 136 * 256) * sizeof(float2))) == cudaSuccess &&
+        (e = cudaMemcpy(pl->cluster_tau, t1, 128 * sizeof(float2), cudaMemcpyDeviceToDevice)) == cudaSuccess)
+        e = cudaMemcpy(static_cast<float2 *>(pl->cluster_tau) + 128, t2, 136 * 256 * sizeof(float2), cudaMemcpyDeviceToDevice);
+    cudaFree(t1);
+    cudaFree(t2);
+    if (st == PACO_OK && e != cudaSuccess) st = fail(PACO_ERR_CUDA, "one-launch form: %s", cudaGetErrorString(e));
+    return st;
 }
 
 } // namespace paco

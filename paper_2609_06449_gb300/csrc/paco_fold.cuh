@@ -184,6 +184,11 @@ __device__ __forceinline__ void fold_dft(cx<R> *v, const Tau &tau)
     for (int i = 0; i < RADIX; ++i) v[i] = u[i];
 }
 
+// With kappa = 0, F2 is plain and w_L^{-k_lo j_lo} a product of its own in FP64 and
+// where F2 is short (at most 8 points: the pass is bound by memory either way,
+// and the plain DFT is the closer one), else folded.
+__host__ __device__ constexpr bool fold_plain(bool fp64, int lgB) { return fp64 || lgB < 4; }
+
 // EPT_: points a thread holds (0: 16, or 32 where a factor needs them).
 template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0>
 struct FoldCfg {
@@ -203,6 +208,7 @@ struct FoldCfg {
     static constexpr int SK = FIRST ? 1 : B * W + (W < PH ? (W - (B * W) % PH + PH) % PH : 0);
     static constexpr int EX = FIRST ? W * SC : A * SK;
     static constexpr bool FP64 = sizeof(R) == 8;
+    static constexpr bool PLAIN2 = TW == 0 && fold_plain(FP64, LGB);   // F2 without factors of its own
     static constexpr bool ROWS = TW && FP64;                      // F1's factors by row (T^r), not by level
     static constexpr int NA = ROWS ? A : A / 2;                   // factors of F1, a column
     static constexpr int NTW = TW == 2 ? (NA + LGB) * W : 0;
@@ -309,7 +315,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
         C *ex = sm + (FIRST ? col * CFG::SC + jlo * CFG::SJ : jlo * W + col);
         if constexpr (TW == 0) {
             plain_dft<A>(v + u * A);
-            if constexpr (CFG::FP64) {
+            if constexpr (CFG::PLAIN2) {
 #pragma unroll
                 for (int k = 1; k < A; ++k) {
                     const V t = __ldg(t1 + k * jlo);         // w_L^{-k_lo j_lo}
@@ -345,7 +351,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
         const C *ex = sm + (FIRST ? col * CFG::SC + klo : klo * CFG::SK + col);
 #pragma unroll
         for (int r = 0; r < B; ++r) v[u * B + r] = ex[r * CFG::SJ];
-        if constexpr (TW == 0 && CFG::FP64) {
+        if constexpr (CFG::PLAIN2) {
             plain_dft<B>(v + u * B);
         } else {
             // factor q of (k_lo, column): entry q A + k_lo after F1's
@@ -422,8 +428,9 @@ template <typename R>
 void fold_pass_args(FoldArgs<R> *a, const FoldKernel &k, const int *f, int n, int i, int t);
 
 // A device table for FoldArgs::tau in mode FoldCfg::TW, 2^lgK columns.
+// kappa = 0 for every column where no_kappa is set.
 template <typename R>
-paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK);
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa = false);
 
 // The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
 // (the row stride); fn == nullptr where none is built.

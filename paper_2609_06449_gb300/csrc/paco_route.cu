@@ -63,11 +63,11 @@ enum TauKind {
     TAU_POWERS      // entry i: w_{K A'}^{-kappa 2^i}
 };
 template <typename R>
-__global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, int lgK)
+__global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, int lgK, bool no_kappa)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    const long long kap = i & ((1ll << lgK) - 1);
+    const long long kap = no_kappa ? 0 : i & ((1ll << lgK) - 1);
     const int q = (int)(i >> lgK);
     long long e;
     int lgM = lgK + lgA;
@@ -85,40 +85,40 @@ __global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, i
 }
 
 template <typename R>
-static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, cudaStream_t s)
+static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, bool no_kappa = false)
 {
     const long long count = (long long)entries << lgK;
-    tau_gen_kernel<R><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(t, count, kind, lgA, lgK);
+    tau_gen_kernel<R><<<(unsigned)((count + 255) / 256), 256>>>(t, count, kind, lgA, lgK, no_kappa);
     return t + count;
 }
 
 // FoldArgs::tau in mode FoldCfg::TW over 2^lgK columns.
 template <typename R>
-paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK)
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa)
 {
     const int A = 1 << k.lgA, B = 1 << k.lgB, lgL = k.lgA + k.lgB;
     const bool fp64 = sizeof(R) == 8;
-    if (mode == 0 && fp64) return gen_table(16, dst, A * B, A * B, 1, 0);
+    if (mode == 0 && fold_plain(fp64, k.lgB)) return gen_table((int)sizeof(cx<R>), dst, A * B, A * B, 1, 0);
     const int nA = fp64 ? A : A / 2;
     const long long cols = 1ll << lgK;
     const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (fp64 && mode == 2 ? (nA + k.lgB) * cols : 0);
     PACO_CUDA_TRY(cudaMalloc(dst, (size_t)count * sizeof(cx<R>)));
     cx<R> *t = static_cast<cx<R> *>(*dst);
     if (mode == 1) {
-        t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, 0) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, 0);
-        tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, 0);
+        t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, no_kappa) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, no_kappa);
+        tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, no_kappa);
     } else {
-        t = tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, 0, 0);
+        t = tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, 0);
         if (fp64 && mode == 2) {
-            t = tau_gen(t, A, TAU_ROWS, k.lgA, lgK, 0);
-            tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK, 0);
+            t = tau_gen(t, A, TAU_ROWS, k.lgA, lgK);
+            tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK);
         }
     }
     PACO_CUDA_TRY(cudaGetLastError());
     return PACO_OK;
 }
 
-template paco_status_t fold_table<float>(void **, const FoldKernel &, int, int);
+template paco_status_t fold_table<float>(void **, const FoldKernel &, int, int, bool);
 
 paco_status_t whole_table(int lgN, void **dst)
 {
@@ -128,7 +128,7 @@ paco_status_t whole_table(int lgN, void **dst)
     for (int i = 1; i < n; ++i) total += 1 << (k[i + 1] - 1);
     PACO_CUDA_TRY(cudaMalloc(dst, (size_t)total * 8));
     cx<float> *t = static_cast<cx<float> *>(*dst);
-    for (int i = 1; i < n; ++i) t = tau_gen(t, 1 << (k[i + 1] - 1), TAU_LEVELS, k[i], 0, 0);
+    for (int i = 1; i < n; ++i) t = tau_gen(t, 1 << (k[i + 1] - 1), TAU_LEVELS, k[i], 0);
     PACO_CUDA_TRY(cudaGetLastError());
     return PACO_OK;
 }

@@ -93,7 +93,8 @@ __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool c
             }
             plain_dft<R>(v + u * R);
         } else {
-            fold_dft<false, float, R>(v + u * R, [&](int q) {
+            // (up to 2^7 points the copy rate leaves room for the closer form)
+            fold_dft<(N <= 128), float, R>(v + u * R, [&](int q) {
                 const float2 t = __ldg(tau + S::tau(I) + q * K + kap);
                 return make_cx<float>(t.x, t.y);
             });

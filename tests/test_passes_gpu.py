@@ -38,7 +38,7 @@ def _run(plan, x, d):
 @pytest.mark.parametrize("d", [-1, 1])
 @pytest.mark.parametrize("l1,l2,b,batch,passes", [
     (2, 2, 2, 3000, 1), (3, 2, 2, 1000, 1), (3, 3, 8, 333, 1), (4, 3, 2, 77, 1), (4, 4, 16, 50, 1), (1, 8, 2, 21, 1),
-    (5, 5, 2, 9, 1), (5, 6, 2, 5, 1), (6, 6, 8, 7, 1), (7, 6, 2, 3, 1), (7, 7, 2, 5, 1), (8, 7, 2, 3, 2), (8, 8, 16, 17, 2),
+    (5, 5, 2, 9, 1), (5, 6, 2, 5, 1), (6, 6, 8, 7, 1), (7, 6, 2, 3, 2), (7, 6, 2, 33, 1), (7, 7, 2, 5, 2), (7, 7, 2, 33, 1), (8, 7, 2, 3, 2), (8, 8, 16, 17, 2),
     (8, 9, 2, 3, 2), (9, 9, 8, 2, 2), (10, 9, 2, 2, 2), (10, 10, 4, 3, 2), (14, 4, 2, 1, 2), (4, 14, 2, 1, 2),
     (11, 10, 2, 2, 3), (12, 10, 2, 2, 3), (11, 12, 2, 1, 3), (12, 12, 16, 1, 3), (13, 12, 2, 1, 3)])
 def test_passes_against_oracle(l1, l2, b, batch, passes, d):
