@@ -23,12 +23,11 @@
 // so far (kappa = column, K of them), and rows are read through pi.
 //
 // Twiddles (TW).  0: kappa = 0 (the first pass; every pass of the 2-D and 3-D
-// forms): plain DFTs, w_L^{-k_lo j_lo} between them.  1: all of the pass's
-// factors come, rounded once from FP64, out of one table of about K L / 2
-// entries, a level's factors being a run in kappa.  2, where that table would
-// not stay in L2 (K L > 2^20): F1's factors and w_{K L}^{-kappa 2^i} are set up
-// per tile in shared memory, rounded once, and a factor of F2 is one more
-// product of such a value with w_L's.
+// forms).  1: all of the pass's factors come, rounded once from FP64, out of one
+// table of about K L / 2 entries, a level's factors being a run in kappa.  2,
+// where that table would not stay in L2 (K L > 2^20): the table holds F1's
+// factors and w_{K L}^{-kappa 2^i}, a tile's part of which goes to shared memory,
+// and a factor of F2 is one more product of such a value with w_L's.
 //
 // The folded butterflies multiply at every level, so the rounding of their
 // factors shows: with all factors as products of rounded values the relative
@@ -56,10 +55,7 @@ struct FoldArgs {
     int lg_tiles;           // log2 of the column tiles of one row block
     int lg_all;             // log2 of the tiles of one transform
     unsigned blk_stride;    // elements between two row blocks
-    const cx<R> *tau;       // the factors: F1's then F2's (TW 0: F2's, TW 2: F2's for kappa = 0)
-    const cx<double> *lo;   // TW 2: w_N^{-r}, r < 2^lo_bits
-    const cx<double> *hi;   //       w_N^{-(r << lo_bits)}
-    int lo_bits;
+    const cx<R> *tau;       // the factors (fold_table)
     int lg_n, lg_k;         // log2 N, log2 K
     int conj;               // 1: the conjugate transform
     int reverse;            // 1: tiles from the last to the first
@@ -245,32 +241,18 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
     const unsigned c0 = (unsigned)(FIRST ? tile : tile & ((1 << a.lg_tiles) - 1)) << CFG::LGW;
     const long long base = boff + (long long)blk * (FIRST ? 0u : a.blk_stride) + c0;
 
-    // TW 2: the columns' factors (exponents of w_N, all below N), used while the
-    // tile is on its way.  With 32 points a thread their table reads go out
+    // TW 2: the columns' factors.  With 32 points a thread their reads go out
     // before the tile's (1024 points 0.93 -> 0.87 ms per 2^28, 512: 0.78 -> 0.75);
-    // with 16 the address work would hold up too many small tiles (256: 0.65, 0.68).
+    // with 16 they would hold up too many small tiles (256: 0.65, 0.68).
     constexpr int NI = (CFG::NTW + NT - 1) / NT;
-    [[maybe_unused]] double2 twl[NI ? NI : 1], twh[NI ? NI : 1];
+    [[maybe_unused]] V twl[NI ? NI : 1];
     [[maybe_unused]] auto load_twiddles = [&] {
 #pragma unroll
         for (int k = 0; k < NI; ++k) {
-            const int e = tid + NT * k, i = e >> CFG::LGW;
-            const unsigned kap = c0 + (e & (W - 1));
-            unsigned x;
-            if (i < CFG::NA) {                               // i = tau_index(n, s)
-                const int lgq = i ? 31 - __clz(i) : 0, lgn = i ? lgq + 2 : 1, s = i ? i - (1 << lgq) : 0;
-                x = ((kap + ((unsigned)s << a.lg_k)) << (CFG::LGA - lgn)) << (a.lg_n - a.lg_k - CFG::LGA);
-            } else {
-                x = (kap << (i - CFG::NA)) << (a.lg_n - a.lg_k - CFG::LGA - CFG::LGB);
-            }
-            if (CFG::NTW % NT == 0 || e < CFG::NTW) {
-                if constexpr (sizeof(R) == 8) {              // rounded once, in the table
-                    twl[k] = __ldg(reinterpret_cast<const double2 *>(a.tau) + CFG::L / 2 + ((unsigned)i << a.lg_k) + kap);
-                    continue;
-                }
-                twl[k] = __ldg(reinterpret_cast<const double2 *>(a.lo + (x & ((1u << a.lo_bits) - 1u))));
-                twh[k] = __ldg(reinterpret_cast<const double2 *>(a.hi + (x >> a.lo_bits)));
-            }
+            const int e = tid + NT * k;
+            if (CFG::NTW % NT == 0 || e < CFG::NTW)
+                twl[k] = __ldg(reinterpret_cast<const V *>(a.tau) + CFG::L / 2 + ((unsigned)(e >> CFG::LGW) << a.lg_k) + c0 +
+                               (e & (W - 1)));
         }
     };
     if constexpr (TW == 2 && CFG::EPT == 32) load_twiddles();
@@ -301,11 +283,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
         if constexpr (CFG::EPT != 32) load_twiddles();
 #pragma unroll
         for (int k = 0; k < NI; ++k)
-            if (CFG::NTW % NT == 0 || tid + NT * k < CFG::NTW) {
-                cx<double> t = make_cx<double>(twl[k].x, twl[k].y);
-                if constexpr (sizeof(R) == 4) t = cmul(t, make_cx<double>(twh[k].x, twh[k].y));
-                tabA[tid + NT * k] = make_cx<R>((R)t.x, (R)t.y);
-            }
+            if (CFG::NTW % NT == 0 || tid + NT * k < CFG::NTW) tabA[tid + NT * k] = make_cx<R>(twl[k].x, twl[k].y);
         __syncthreads();
     }
 #pragma unroll

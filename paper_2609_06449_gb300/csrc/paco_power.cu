@@ -1,6 +1,7 @@
 // paco_power.cu -- the kernels of paco_power.cuh by stage length.  The tiles
 // and the factors A * B are the stage kernels', so that a thread's partial sums
 // cover the same results.
+#include "paco_plan.h"
 #include "paco_power.cuh"
 
 namespace paco {
@@ -31,6 +32,22 @@ static PowerKernel pick(int lgL, int lgC)
     case 10: return lgC >= 3 ? kernel_of<5, 5, 3, FIRST>() : PowerKernel();
     default: return PowerKernel();
     }
+}
+
+__global__ void power_table_kernel(const cx<float> *w, cx<float> *out, int lgL)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x, s = 1 << ((lgL + 1) / 2);
+    if (r >= 1 << lgL) return;
+    const cx<float> lo = w[r & (s - 1)], hi = w[r & ~(s - 1)];
+    out[r] = lgL > 6 ? st::mul<1>(lo, hi) : st::mul<0>(lo, hi);
+}
+
+paco_status_t power_table(const cx<float> *w, int lgL, void **dst)
+{
+    PACO_CUDA_TRY(cudaMalloc(dst, (size_t)8 << lgL));
+    power_table_kernel<<<((1 << lgL) + 255) / 256, 256>>>(w, static_cast<cx<float> *>(*dst), lgL);
+    PACO_CUDA_TRY(cudaGetLastError());
+    return PACO_OK;
 }
 
 PowerKernel power_kernel(bool first, int lgL, int lgC) { return first ? pick<true>(lgL, lgC) : pick<false>(lgL, lgC); }

@@ -14,6 +14,7 @@
 // instructions a point on run-time strides and twiddle products.
 #pragma once
 
+#include "../../include/paco.h"
 #include "paco_fold.cuh"
 
 namespace paco {
@@ -28,7 +29,7 @@ struct PowerArgs {
     int rev_bits, rev_t;    // row map of j_lo: pi over rev_bits bits (0: natural rows)
     int crev_bits, crev_t;  // Phase I: row pi(c) of column c
     int lg_all;             // log2 of the tiles of one transform (blockIdx.x = transform, tile)
-    const cx<float> *twL;   // w_L^{-r}, r < L
+    const cx<float> *twL;   // w_L^{-r}, r < L, as the stage kernels' product of two factors (power_table)
     const cx<float> *lo;    // w_N^{-r}, r < 2^lo_bits
     const cx<float> *hi;    // w_N^{-(r << lo_bits)}
     int lo_bits;
@@ -149,7 +150,6 @@ struct PowerCfg {
     static constexpr int LGA = LGA_, LGB = LGB_, LGW = LGW_;
     static constexpr bool FIRST = FIRST_;
     static constexpr int A = 1 << LGA, B = 1 << LGB, W = 1 << LGW, L = A * B;
-    static constexpr int LG_SL = (LGA + LGB + 1) / 2, SL = 1 << LG_SL;   // w_L^{-r} = w[r mod SL] w[r / SL * SL]
     static constexpr int EPT = (LGA == 5 || LGB == 5) ? 32 : 16;   // points a thread holds
     static constexpr int NT = L * W / EPT;
     static constexpr int U1 = EPT / A, U2 = EPT / B;               // sequences a thread, F1 and F2
@@ -217,10 +217,8 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_power_kernel(const __
         ex[0] = v[u * A];
 #pragma unroll
         for (int k = 1; k < A; ++k) {
-            const int r = k * jlo;
-            const float2 l = __ldg(tw + (r & (CFG::SL - 1))), h = __ldg(tw + (r & ~(CFG::SL - 1)));
-            const C w = st::mul<(CFG::L > 64)>(make_cx<float>(l.x, l.y), make_cx<float>(h.x, h.y));
-            ex[FIRST ? k : k * CFG::SK] = st::mul<0>(v[u * A + k], w);
+            const float2 t = __ldg(tw + k * jlo);
+            ex[FIRST ? k : k * CFG::SK] = st::mul<0>(v[u * A + k], make_cx<float>(t.x, t.y));
         }
     }
     // w_N^{-k_lo c} (read before the barrier: its two table reads overlap the others' F1)
@@ -309,5 +307,9 @@ struct PowerKernel {
 // The kernel of a stage of length 2^lgL over 2^lgC columns; fn == nullptr
 // where none is built.
 PowerKernel power_kernel(bool first, int lgL, int lgC);
+
+// PowerArgs::twL from w_L^{-r} (r < L = 2^lgL): entry r is the product
+// w[r mod S] w[r / S * S], S = 2^ceil(lgL / 2), that the stage kernels take.
+paco_status_t power_table(const cx<float> *w, int lgL, void **dst);
 
 } // namespace paco

@@ -38,7 +38,6 @@ struct Route {
     PowerKernel pk[2];              // the stages of the weighted power (fn == nullptr: the stage kernels)
     PowerArgs pa[2];
     void *tw[MAX_PASSES + 2] = {};     // the factors of every pass, w_L^{-r} of the two stages
-    void *lo64 = nullptr, *hi64 = nullptr;
 };
 
 // pi over `bits` bits with digits of t bits (host copy of digit_reverse).
@@ -51,8 +50,6 @@ void route_destroy(Route *r)
 {
     if (!r) return;
     for (void *p : r->tw) cudaFree(p);
-    cudaFree(r->lo64);
-    cudaFree(r->hi64);
     delete r;
 }
 
@@ -101,7 +98,7 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
     if (mode == 0 && fold_plain(fp64, k.lgB)) return gen_table((int)sizeof(cx<R>), dst, A * B, A * B, 1, 0);
     const int nA = fp64 ? A : A / 2;
     const long long cols = 1ll << lgK;
-    const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (fp64 && mode == 2 ? (nA + k.lgB) * cols : 0);
+    const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (mode == 2 ? (nA + k.lgB) * cols : 0);
     PACO_CUDA_TRY(cudaMalloc(dst, (size_t)count * sizeof(cx<R>)));
     cx<R> *t = static_cast<cx<R> *>(*dst);
     if (mode == 1) {
@@ -109,8 +106,8 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
         tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, no_kappa);
     } else {
         t = tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, 0);
-        if (fp64 && mode == 2) {
-            t = tau_gen(t, A, TAU_ROWS, k.lgA, lgK);
+        if (mode == 2) {
+            t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK) : tau_gen(t, nA, TAU_LEVELS, 0, lgK);
             tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK);
         }
     }
@@ -169,21 +166,10 @@ static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, c
 {
     const FoldKernel &k = r->k[i];
     fold_pass_args(a, k, f, n, i, t);
-    a->lo_bits = pl->twN_lo_bits;
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    paco_status_t st = fold_table<R>(&r->tw[i], k, r->twmode[i], a->lg_k);
+    const paco_status_t st = fold_table<R>(&r->tw[i], k, r->twmode[i], a->lg_k);
     a->tau = static_cast<const cx<R> *>(r->tw[i]);
-    if (st != PACO_OK || r->twmode[i] != 2 || sizeof(R) == 8) return st;
-    // w_N^{-r} in FP64, two levels
-    if (!r->lo64) {
-        const long long nlo = 1LL << pl->twN_lo_bits;
-        if ((st = gen_table(16, &r->lo64, pl->N, nlo, 1, 0)) != PACO_OK ||
-            (st = gen_table(16, &r->hi64, pl->N, pl->N / nlo, nlo, 0)) != PACO_OK)
-            return st;
-    }
-    a->lo = static_cast<const cx<double> *>(r->lo64);
-    a->hi = static_cast<const cx<double> *>(r->hi64);
-    return PACO_OK;
+    return st;
 }
 
 // Stage i of the weighted power over the plan's factors.
@@ -205,7 +191,10 @@ static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerK
     a->lo_bits = pl->twN_lo_bits;
     a->n_mask = (unsigned)(pl->N - 1);
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    const paco_status_t st = gen_table(8, tw, 1LL << lgL, 1LL << lgL, 1, 0);
+    void *w = nullptr;
+    paco_status_t st = gen_table(8, &w, 1LL << lgL, 1LL << lgL, 1, 0);
+    if (st == PACO_OK) st = power_table(static_cast<const cx<float> *>(w), lgL, tw);
+    cudaFree(w);
     a->twL = static_cast<const cx<float> *>(*tw);
     return st;
 }
@@ -248,7 +237,7 @@ static paco_status_t tc_setup(paco_plan *pl, Route *r, int lgN)
         if (!r->k[i].fn) return PACO_OK;
         TcPassArgs &a = r->t[i];
         fold_pass_args(&a.f, r->k[i], f, n, i, t);
-        a.f.lo_bits = pl->twN_lo_bits;
+        a.lo_bits = pl->twN_lo_bits;
         a.lo = static_cast<const cx<float> *>(pl->twN_lo);
         a.hi = static_cast<const cx<float> *>(pl->twN_hi);
         a.frag = static_cast<const uint4 *>(pl->tc);
@@ -366,7 +355,7 @@ paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir,
         a.mult = terms ? terms->ld_mult : 1.f;
         a.scale = terms ? terms->ld_scale : nullptr;
         return launch(pl, r.whole.fn, &a, (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta, r.whole.threads,
-                      r.whole.smem, true, stream);
+                      r.whole.smem, false, stream);
     }
     if (pl->form) {
         for (int i = 0; i < r.n; ++i) {

@@ -31,8 +31,9 @@ namespace paco {
 struct TcPassArgs {
     FoldArgs<float> f;      // strides, row maps (rowK aside)
     const cx<float> *twL;   // w_L^{-r}, r < L
-    const cx<float> *lo;    // w_N^{-r}, r < 2^f.lo_bits
-    const cx<float> *hi;    // w_N^{-(r << f.lo_bits)}
+    const cx<float> *lo;    // w_N^{-r}, r < 2^lo_bits
+    const cx<float> *hi;    // w_N^{-(r << lo_bits)}
+    int lo_bits;
     const uint4 *frag;      // the matrix fragments (tc_table_create)
 };
 
@@ -183,8 +184,8 @@ __global__ void __launch_bounds__(CFG::NT, CFG::CTAS) paco_tcpass_kernel(const _
             const unsigned kap = c0 + (e & (W - 1));
             const int r = e >> LGW;
             const unsigned ex = r < A ? (kap * (unsigned)r) << (sh - 4) : (kap * (unsigned)(r - A)) << (sh - lgL);
-            const float2 l = __ldg(reinterpret_cast<const float2 *>(args.lo + (ex & ((1u << a.lo_bits) - 1u))));
-            const float2 h = __ldg(reinterpret_cast<const float2 *>(args.hi + (ex >> a.lo_bits)));
+            const float2 l = __ldg(reinterpret_cast<const float2 *>(args.lo + (ex & ((1u << args.lo_bits) - 1u))));
+            const float2 h = __ldg(reinterpret_cast<const float2 *>(args.hi + (ex >> args.lo_bits)));
             rows[e] = cmul(make_cx<float>(l.x, l.y), make_cx<float>(h.x, h.y));
         }
     }

@@ -142,8 +142,6 @@ __global__ void __launch_bounds__(NT, (EPT == 16 ? 1024 : 512) / NT) paco_whole_
 {
     using CFG = WholeCfg<LG, EPT, NT>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    grid_launch_dependents();
-    grid_wait();
     const long long t0 = (long long)blockIdx.x * CFG::G;
     const float f = a.scale ? a.mult * (float)__ldg(a.scale) : a.mult;
     whole_step<CFG, EPT, NT, 0>(
