@@ -3,17 +3,17 @@
 
 Default workload (the headline): one complex64 1-D DFT of N = 2^28 as
 N1 = N2 = 2^14, radix b = 4, p = 64 virtual slabs, forward (w^{-kj}); input
-Re/Im i.i.d. U[-1, 1) from seed (rank).  One step = one pass of the whole
-path: Phase I with the fused twiddle + digit-reversal redistribution
-(stage 1), then Phase III (stage 2), exactly the two launches paco_execute
-makes.  The input (2 GiB) is larger than L2, so no flush is needed between
+Re/Im i.i.d. U[-1, 1) from seed (rank).  One step = one paco_execute, the
+whole path: Phase I with the digit-reversal redistribution in its stores, then
+Phase III, in the passes the plan chose (paco_plan_info.passes launches).  The
+input (2 GiB) is larger than L2, so no flush is needed between
 steps.  The same line carries the tensor-core sub-DFT forms (BF16x3 split,
 FP16 per-block scaled) timed on the same transform, each with its relative
 L2 error against the FP64 oracle.
 
 Reported: 5 N log2 N GFLOP/s (whole job), effective HBM GB/s (32 N bytes per
-step: two reads and two writes of N complex64), the dominant kernel's
-roofline against the measured copy bandwidth, an end-to-end number through
+step: two reads and two writes of N complex64), the mean pass's roofline
+against the measured copy bandwidth, an end-to-end number through
 paco_execute_host with pinned host buffers, the CPU oracle on a bounded
 sample, SM clocks sampled during the timed region, and cuFFT on the same
 input as context.
@@ -274,10 +274,10 @@ def workload_config(args):
     }
 
 
-def captured_traffic(stage: str, N1: int, N2: int, b: int, p: int, dtype: str, dir: int):
-    """DRAM bytes per launch of the panel kernel from the committed ncu
-    capture (profiles/roofline_traffic.json), or None when the workload differs
-    or the kernel source changed since the counters were taken."""
+def captured_traffic(N1: int, N2: int, b: int, p: int, dtype: str, dir: int):
+    """DRAM bytes per launch (mean of the passes) from the committed ncu capture
+    (profiles/roofline_traffic.json), or None when the workload differs or the
+    kernel source changed since the counters were taken."""
     import hashlib
     if (N1, N2, b, p, dtype, dir) != (1 << 14, 1 << 14, 4, 64, "c64", -1):
         return None
@@ -286,13 +286,14 @@ def captured_traffic(stage: str, N1: int, N2: int, b: int, p: int, dtype: str, d
             rec = json.load(fh)
         csrc = os.path.join(ROOT, "paper_2609_06449_gb300", "csrc")
         h = hashlib.sha256()
-        for name in ("paco_panel.cuh", "paco_common.cuh"):
+        for name in ("paco_fold.cuh", "paco_common.cuh"):
             with open(os.path.join(csrc, name), "rb") as fh:
                 h.update(fh.read())
         if h.hexdigest()[:16] != rec["source_sha16"]:
             return None
-        return float(rec["traffic_bytes_per_launch"][stage])
-    except (OSError, KeyError, ValueError):
+        per = rec["traffic_bytes_per_launch"]
+        return float(sum(per) / len(per))
+    except (OSError, KeyError, TypeError, ValueError):
         return None
 
 
@@ -402,6 +403,11 @@ def cpu_leg(args, rank, world, dtype="c64", lg=None, threads=None):
                           f"FP64 recursive radix-2 oracle, {nt} thread(s), {per:.2f} s each"}
     except Exception as e:  # report, do not hide
         return {"value": None, "unit": "GFLOP/s", "cores": 0, "kind": "oracle", "sample": f"failed: {e}"}
+
+
+def exec_launches(info):
+    """Kernel launches of one paco_execute on this plan."""
+    return int(info.passes) or (1 if info.fused_cluster else 2 + sum(info.stage_split))
 
 
 def hbm_roofline(kernel, bytes_per_launch, ms_per_launch, traffic=None):
@@ -521,32 +527,21 @@ def run_other(args, ranks, local):
         xh = torch.from_numpy(uniform(N, rank, np.complex128)).pin_memory()
         x = xh.cuda()
         y = torch.empty_like(x)
-        ev = [[torch.cuda.Event(enable_timing=True) for _ in range(3)] for _ in range(K)]
-
-        def step2(k=[0]):
-            i = k[0] % K
-            ev[i][0].record(stream)
-            plan.execute_stage1(x, y, args.dir, stream)
-            ev[i][1].record(stream)
-            plan.execute_stage2(y, y, args.dir, stream)
-            ev[i][2].record(stream)
-            k[0] += 1
+        launches = exec_launches(plan.info)
         for _ in range(W):
             plan.execute(x, y, args.dir, stream)
-        tot, per, clocks = timed(step2)
+        tot, per, clocks = timed(lambda: plan.execute(x, y, args.dir, stream))
         plan.check()
-        s1 = statistics.mean(ev[k][0].elapsed_time(ev[k][1]) for k in range(K))
-        s2 = statistics.mean(ev[k][1].elapsed_time(ev[k][2]) for k in range(K))
         flop = 5.0 * N * 27
         ms = mor(tot) / K
         fp64_peak, fp64_src = fp64_peak_measured(paco, local)
-        dom_ms = max(s1, s2)
+        step_ms = statistics.mean(per)
         ho = torch.empty_like(xh).pin_memory()
         di = torch.empty_like(x)
         e2e = None if args.no_e2e else e2e_host(lambda: plan.execute_host(xh, ho, di, y, args.dir, stream), max(args.e2e_steps, 1), stream,
                        flop / 1e9, "GFLOP/s", N * 16, N * 16, "paco_execute_host (pinned host buffers)", mor,
                        world, ranks.barrier)
-        hr = hbm_roofline("stage1" if s1 >= s2 else "stage2", 32.0 * N, dom_ms)
+        hr = hbm_roofline(f"paco_fold_kernel (mean of {launches} passes)", 32.0 * N, step_ms / launches)
         import oracle
         plan.execute(x, y, args.dir, stream)
         torch.cuda.synchronize()
@@ -562,15 +557,15 @@ def run_other(args, ranks, local):
                                         + ("forward" if args.dir == -1 else "conjugate"), "dir": args.dir,
                             "N1": N1, "N2": N2, "b": 2, "p": 128, "batch": 1,
                             "input": "Re, Im i.i.d. U[-1,1), seed = rank", "l2": "inputs larger than L2"},
-                    stage_ms={"stage1": s1, "stage2": s2}, hbm_gbs_effective=64.0 * N * world / (ms * 1e-3) / 1e9,
+                    launches_per_step=launches, hbm_gbs_effective=64.0 * N * world / (ms * 1e-3) / 1e9,
                     accuracy=acc, context=cufft_context(x, N, 1, flop),
                     roofline={"bound": "alu", "kernel": hr["kernel"],
-                              "achieved": flop / 2 / (dom_ms * 1e-3) / 1e12, "peak": fp64_peak / 1e3,
-                              "unit": "TFLOP/s (nominal 5N log2 N flops, half per stage)",
+                              "achieved": flop / (step_ms * 1e-3) / 1e12, "peak": fp64_peak / 1e3,
+                              "unit": "TFLOP/s (nominal 5N log2 N flops)",
                               "peak_source": fp64_src,
-                              "frac": flop / 2 / (dom_ms * 1e-3) / 1e12 / (fp64_peak / 1e3),
+                              "frac": flop / (step_ms * 1e-3) / 1e12 / (fp64_peak / 1e3),
                               "traffic": None, "hbm": hr},
-                    e2e=e2e, cpu_baseline=cpu_leg(args, rank, world, "c128"), gpu_launches=2 * K, clocks=clocks)
+                    e2e=e2e, cpu_baseline=cpu_leg(args, rank, world, "c128"), gpu_launches=launches * K, clocks=clocks)
     elif wl == "C":
         if args.small:
             e = uneven_lengths(count=1024, seed=0, lo=8, hi=20, total_log2=26)
@@ -641,10 +636,10 @@ def run_other(args, ranks, local):
             ms = mor(tot) / K
             torch.cuda.synchronize()
             err = rel_l2_vs_oracle(y[:N].cpu().numpy(), xh[:N].numpy())
-            split = tuple(pl.info.stage_split)
+            launches = exec_launches(pl.info)
             forms[name] = {"ms_per_step": ms, "value": flop * world / (ms * 1e-3) / 1e9, "unit": "GFLOP/s",
-                           "rel_l2_transform0": err, "dominant_launch_ms": statistics.mean(per) / 2,
-                           "stage_split": list(split), "launches_per_step": 2 + sum(split)}
+                           "rel_l2_transform0": err, "mean_launch_ms": statistics.mean(per) / launches,
+                           "launches_per_step": launches}
             if name == "bf16x3":
                 clocks = ck
             pl.close()
@@ -660,9 +655,8 @@ def run_other(args, ranks, local):
                             "input": "log-uniform magnitudes 1e-4..1e4, uniform phases, seed = 100*rank + i",
                             "l2": "inputs larger than L2"},
                     forms=forms, context=cufft_context(x, N, B, flop),
-                    roofline=hbm_roofline(f"stage kernel ({head})" + (", two passes per stage"
-                                                                       if sum(forms[head]["stage_split"]) else ""),
-                                          16.0 * N * B, forms[head]["dominant_launch_ms"]),
+                    roofline=hbm_roofline(f"pass kernel ({head}), mean of {forms[head]['launches_per_step']} passes",
+                                          16.0 * N * B, forms[head]["mean_launch_ms"]),
                     e2e=None, cpu_baseline=cpu_leg(args, rank, world),
                     gpu_launches=K * sum(f["launches_per_step"] for f in forms.values()), clocks=clocks)
         # e2e for the form of the line's value
@@ -747,7 +741,7 @@ def run_other(args, ranks, local):
         sp = [statistics.mean(ev[k][j].elapsed_time(ev[k][j + 1]) for k in range(K)) for j in range(3)]
         flop = 5.0 * N * 2 * lg
         ms = mor(tot) / K
-        # the fused two-pass path on the same transform, for the ratio
+        # paco_execute on the same transform, for the ratio
         yf = torch.empty_like(x)
         ftot, fper = time_steps(lambda: plan.execute(x, yf, -1, stream), K, 3, stream)
         line = dict(base, value=flop * world / (ms * 1e-3) / 1e9, unit="GFLOP/s", higher_is_better=True,
@@ -768,7 +762,7 @@ def run_other(args, ranks, local):
         x = xh.cuda()
         y = torch.empty_like(x)
         plan = paco.Plan(N1, N2, 2, B, paco.C64, dims=3, N3=N3)
-        launches = 2 + sum(plan.info.stage_split)
+        launches = exec_launches(plan.info)
         for _ in range(W):
             plan.execute(x, y, -1, stream)
         tot, per, clocks = timed(lambda: plan.execute(x, y, -1, stream))
@@ -789,14 +783,14 @@ def run_other(args, ranks, local):
                                         "output axes reversed",
                             "N1": N1, "N2": N2, "N3": N3, "batch": B, "input": "Re, Im i.i.d. U[-1,1), seed = rank",
                             "l2": "inputs larger than L2"},
-                    stage_split=list(plan.info.stage_split), launches_per_step=launches,
+                    launches_per_step=launches,
                     hbm_gbs_effective=16.0 * launches * N * B * world / (ms * 1e-3) / 1e9,
                     accuracy={"rel_l2_vs_cufft_fftn": diff,
                               "measured_on": "the whole output vs torch.fft.fftn (parity with the oracle is in the tests)"},
                     context={"cufft_fftn_ms_per_step": cms, "cufft_gflops": flop / (cms * 1e-3) / 1e9,
                              "source": "torch.fft.fftn over the three axes (cuFFT), same input, median of %d"
                                        % min(K, 20)},
-                    roofline=hbm_roofline(f"stage kernels, {launches} passes (Phase III split over the "
+                    roofline=hbm_roofline(f"paco_fold_kernel, mean of {launches} passes (Phase III split over the "
                                           f"{N2} x {N3} planes)", 16.0 * N * B, statistics.mean(per) / launches),
                     e2e=None if args.no_e2e else e2e_host(lambda: plan.execute_host(xh, ho, di, y, -1, stream),
                                                           max(args.e2e_steps, 1), stream, flop / 1e9, "GFLOP/s",
@@ -912,45 +906,39 @@ def main():
     stream = torch.cuda.current_stream()
 
     for _ in range(max(args.warmup, 3)):
-        plan.execute_stage1(x, out, args.dir, stream)
-        plan.execute_stage2(out, out, args.dir, stream)
+        plan.execute(x, out, args.dir, stream)
     torch.cuda.synchronize()
     plan.check()
 
     K = args.steps
-    ev = [[torch.cuda.Event(enable_timing=True) for _ in range(3)] for _ in range(K)]
+    launches = exec_launches(plan.info)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
     sampler = ClockSampler(local)
     sampler.start()
     time.sleep(0.3)
     barrier()
     torch.cuda.synchronize()
     t_begin = time.time()
-    for k in range(K):
-        ev[k][0].record(stream)
-        plan.execute_stage1(x, out, args.dir, stream)
-        ev[k][1].record(stream)
-        plan.execute_stage2(out, out, args.dir, stream)
-        ev[k][2].record(stream)
+    ev[0].record(stream)
+    for _ in range(K):
+        plan.execute(x, out, args.dir, stream)
+    ev[1].record(stream)
     torch.cuda.synchronize()
     t_end = time.time()
     barrier()
     clocks = sampler.stop(t_begin, t_end)
     plan.check()
 
-    total_ms = ev[0][0].elapsed_time(ev[K - 1][2])
-    s1 = [ev[k][0].elapsed_time(ev[k][1]) for k in range(K)]
-    s2 = [ev[k][1].elapsed_time(ev[k][2]) for k in range(K)]
+    total_ms = ev[0].elapsed_time(ev[1])
     flop = 5.0 * N * lgN
     value = ranks.job_value(flop / 1e9, total_ms / K * 1e-3)
     ms_step = max_over_ranks(total_ms) / K
     hbm_eff = 4.0 * N * esize * world / (ms_step * 1e-3) / 1e9
 
-    avg1, avg2 = statistics.mean(s1), statistics.mean(s2)
-    dom, dom_ms, dom_key = ("stage1 (Phase I + fused PARA-CO-DRP)", avg1, "stage1") if avg1 >= avg2 else \
-        ("stage2 (Phase III)", avg2, "stage2")
-    traffic = captured_traffic(dom_key, N1, N2, args.b, args.p, args.dtype, args.dir)
+    pass_ms = total_ms / K / launches             # mean launch
+    traffic = captured_traffic(N1, N2, args.b, args.p, args.dtype, args.dir)
     bytes_per_launch = 2.0 * N * esize            # read N + write N elements
-    achieved = bytes_per_launch / (dom_ms * 1e-3) / 1e9
+    achieved = bytes_per_launch / (pass_ms * 1e-3) / 1e9
     peak, peak_src = measured_peak_hbm()
 
     # end to end: host buffers through paco_execute_host (H2D + execute + D2H)
@@ -995,12 +983,12 @@ def main():
             "dtype": "f32" if args.dtype == "c64" else "f64", "data": "synthetic",
             "config": workload_config(args),
             "hbm_gbs_effective": hbm_eff,
-            "stage_ms": {"stage1": avg1, "stage2": avg2},
-            "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak,
+            "launches_per_step": launches,
+            "roofline": {"bound": "hbm", "kernel": f"paco_fold_kernel (mean of {launches} passes)", "achieved": achieved, "peak": peak,
                          "peak_source": peak_src, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": traffic,
                          "algorithmic_bytes_per_launch": bytes_per_launch},
-            "e2e": e2e, "cpu_baseline": cpu, "cpu_baseline_1core": cpu1, "gpu_launches": 2 * K,
+            "e2e": e2e, "cpu_baseline": cpu, "cpu_baseline_1core": cpu1, "gpu_launches": launches * K,
             "clocks": clocks, "tc_split": tc, "context": context,
         }
         print(json.dumps(line), flush=True)

@@ -176,17 +176,22 @@ paco_status_t paco_plan_info(const paco_plan_t *plan, paco_plan_info_t *info);
  * its stores (the PARA-CO-DRP_b middle stage, Sect. 4.2), then Phase III
  * (LocalFFT, input layout) reading that layout.  `in` and `out` are device
  * buffers of batch*N elements of the plan's dtype; `out` also holds the
- * intermediate W = Z-hat (Eq. (17)) between the two kernels, so no scratch
- * is used.  in == out, or overlapping buffers, return PACO_ERR_ALIASING.
+ * intermediate between the kernels.  Plans with no stage option set run the
+ * composition over factors of N chosen for the machine (paco_plan_info.passes
+ * launches: whole transforms of complex64 up to 2^14 points in one, else two
+ * to four passes, the first with the redistribution in its stores, the others
+ * in place in `out`); the others run the plan's own two stages, W = Z-hat
+ * (Eq. (17)) between them.  The launches may be programmatically dependent:
+ * they wait for the preceding kernels before they touch `in` or `out`.  in == out, or overlapping buffers, return PACO_ERR_ALIASING.
  * batch = 0 is a no-op.  Asynchronous on `stream`.  A complex64 plan with
  * N1 = N2 = 256, p = 4 or 8 and batch <= 16 (where one launch is faster than
  * two) runs as ONE launch (paco_plan_info.fused_cluster): a thread-block
  * cluster of K = 16 CTAs per transform (8 where the GPU cannot host a
  * 16-CTA cluster), processor q of Sect. 2 being the K/p CTAs that hold its
  * slab -- Phase I on the input columns in shared memory, then PARA-CO-DRP_b
- * (Sect. 4.2, App. C.5) as one all-to-all of asynchronous stores into the
- * other CTAs' shared memory (N/p^2 items per ordered pair of processors, a
- * CTA's items for itself kept in the CTA), then Phase
+ * (Sect. 4.2, App. C.5) as one all-to-all of bulk copies into the other CTAs'
+ * shared memory (N/p^2 items per ordered pair of processors, a CTA's items
+ * for itself kept in the CTA), then Phase
  * III on its output columns; W never reaches global memory.  The launch
  * allows programmatic dependent launch (it waits for the preceding kernels
  * before it reads `in`).  A device-side wait of this form that gives up after
@@ -451,7 +456,9 @@ paco_status_t paco_plan_batched_config(const paco_plan_t *plan, int64_t length, 
  * PACO_ERR_TIMEOUT, and the CUDA context stays usable.  In the one-launch
  * cluster form (fused_cluster = 1) wait_bias > 0 makes each CTA's transaction
  * barrier expect 8 * wait_bias bytes that never come, so its 2 s wait runs
- * out the same way.  Set both to 0 for normal use.  Returns
+ * out the same way.  With the hook set, paco_execute of a plan with panel
+ * stages runs those instead of its passes (which wait on nothing of that
+ * kind).  Set both to 0 for normal use.  Returns
  * PACO_ERR_INVALID_ARG for a NULL plan.
  */
 paco_status_t paco_debug_set_waits(paco_plan_t *plan, unsigned spin_limit, unsigned wait_bias);

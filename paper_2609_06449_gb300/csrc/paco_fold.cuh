@@ -205,6 +205,12 @@ struct FoldCfg {
     static constexpr int EX = FIRST ? W * SC : A * SK;
     static constexpr bool FP64 = sizeof(R) == 8;
     static constexpr bool PLAIN2 = TW == 0 && fold_plain(FP64, LGB);   // F2 without factors of its own
+    // F1's factors read ahead of the tile, with 16 points a thread (2^28 points: 128
+    // 0.648 -> 0.610 ms).  With 32 they cost more than they hide: 512 0.66 -> 0.72;
+    // 1024 0.853 -> 0.834, but one 2^20 12.3 -> 14.3 us.
+    static constexpr bool AHEAD = TW == 1 && !FP64 && EPT == 16;
+    // F2's butterflies in the closer form (bfly), but where the error has room
+    static constexpr bool DIRECT = TW != 1 && !FP64 && (FIRST || TW == 2 || LGB < 5);
     static constexpr bool ROWS = TW && FP64;                      // F1's factors by row (T^r), not by level
     static constexpr int NA = ROWS ? A : A / 2;                   // factors of F1, a column
     static constexpr int NTW = TW == 2 ? (NA + LGB) * W : 0;
@@ -257,6 +263,14 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
     };
     if constexpr (TW == 2 && CFG::EPT == 32) load_twiddles();
 
+    [[maybe_unused]] V ahead[CFG::AHEAD ? U1 : 1][CFG::AHEAD ? A / 2 : 1];
+    if constexpr (CFG::AHEAD) {
+#pragma unroll
+        for (int u = 0; u < U1; ++u)
+#pragma unroll
+            for (int q = 0; q < A / 2; ++q)
+                ahead[u][q] = __ldg(reinterpret_cast<const V *>(a.tau) + c0 + ((tid + NT * u) & (W - 1)) + ((unsigned)q << a.lg_k));
+    }
     if constexpr (PDL) grid_wait();
     // ---- F1
     C v[CFG::EPT];
@@ -304,6 +318,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             t1 += c0 + col;
             auto f1 = [&](int q) {
                 if constexpr (TW == 2) return tabA[q * W + col];
+                if constexpr (CFG::AHEAD) return make_cx<R>(ahead[u][q].x, ahead[u][q].y);
                 const V t = __ldg(t1 + ((unsigned)q << a.lg_k));
                 return make_cx<R>(t.x, t.y);
             };
@@ -336,7 +351,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             const V *t2 = reinterpret_cast<const V *>(a.tau);
             if constexpr (TW == 1) t2 += c0 + col + ((unsigned)(CFG::NA + klo) << a.lg_k);
             else t2 += klo;
-            fold_dft<TW != 1 && !CFG::FP64, R, B>(v + u * B, [&](int q) {
+            fold_dft<CFG::DIRECT, R, B>(v + u * B, [&](int q) {
                 const V t = __ldg(t2 + (TW == 1 ? (unsigned)(q * A) << a.lg_k : (unsigned)(q * A)));
                 const C w = make_cx<R>(t.x, t.y);
                 if constexpr (TW != 2) return w;

@@ -59,8 +59,12 @@ enum TauKind {
     TAU_ROWS,       // entry r: w_{K A'}^{-kappa r}
     TAU_POWERS      // entry i: w_{K A'}^{-kappa 2^i}
 };
+struct Roots {
+    const cx<double> *lo = nullptr, *hi = nullptr;   // (nullptr: by sincospi)
+    int lg = 0, lo_bits = 0;                         // of w_{2^lg}
+};
 template <typename R>
-__global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, int lgK, bool no_kappa)
+__global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, int lgK, bool no_kappa, Roots roots)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
@@ -76,16 +80,34 @@ __global__ void tau_gen_kernel(cx<R> *out, long long count, int kind, int lgA, i
     } else {
         e = kind == TAU_ROWS ? kap * q : kap << q;
     }
+    if (roots.lo) {
+        // the product of two FP64 roots, rounded once (a tenth of sincospi's work)
+        const unsigned x = (unsigned)(e << (roots.lg - lgM));
+        const cx<double> w = cmul(roots.lo[x & ((1u << roots.lo_bits) - 1u)], roots.hi[x >> roots.lo_bits]);
+        out[i] = make_cx<R>((R)w.x, (R)w.y);
+        return;
+    }
     double sn, cs;
     sincospi(2.0 * (double)e / (double)(1ll << lgM), &sn, &cs);
     out[i] = make_cx<R>((R)cs, (R)(-sn));
 }
 
+// lo[r] = w^{-r}, r < 2^lo_bits, then hi[r] = w^{-(r << lo_bits)}, w = w_{2^lg}.
+__global__ void roots_gen_kernel(cx<double> *out, int lg, int lo_bits)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, nlo = 1 << lo_bits;
+    if (i >= nlo + (1 << (lg - lo_bits))) return;
+    const long long e = i < nlo ? i : (long long)(i - nlo) << lo_bits;
+    double sn, cs;
+    sincospi(2.0 * (double)e / (double)(1ll << lg), &sn, &cs);
+    out[i] = make_cx<double>(cs, -sn);
+}
+
 template <typename R>
-static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, bool no_kappa = false)
+static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, bool no_kappa = false, const Roots &roots = Roots())
 {
     const long long count = (long long)entries << lgK;
-    tau_gen_kernel<R><<<(unsigned)((count + 255) / 256), 256>>>(t, count, kind, lgA, lgK, no_kappa);
+    tau_gen_kernel<R><<<(unsigned)((count + 255) / 256), 256>>>(t, count, kind, lgA, lgK, no_kappa, roots);
     return t + count;
 }
 
@@ -99,16 +121,31 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
     const int nA = fp64 ? A : A / 2;
     const long long cols = 1ll << lgK;
     const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (mode == 2 ? (nA + k.lgB) * cols : 0);
-    PACO_CUDA_TRY(cudaMalloc(dst, (size_t)count * sizeof(cx<R>)));
+    // FP32 tables of many entries: FP64 roots of w_{K L} behind the table
+    Roots roots;
+    size_t bytes = ((size_t)count * sizeof(cx<R>) + 15) & ~(size_t)15;
+    const bool by_roots = !fp64 && mode != 0 && !no_kappa;
+    if (by_roots) {
+        roots.lg = lgK + lgL;
+        roots.lo_bits = (roots.lg + 1) / 2;
+    }
+    const int nroots = by_roots ? (1 << roots.lo_bits) + (1 << (roots.lg - roots.lo_bits)) : 0;
+    PACO_CUDA_TRY(cudaMalloc(dst, bytes + (size_t)nroots * sizeof(cx<double>)));
+    if (by_roots) {
+        cx<double> *q = reinterpret_cast<cx<double> *>(static_cast<char *>(*dst) + bytes);
+        roots_gen_kernel<<<(nroots + 255) / 256, 256>>>(q, roots.lg, roots.lo_bits);
+        roots.lo = q;
+        roots.hi = q + (1 << roots.lo_bits);
+    }
     cx<R> *t = static_cast<cx<R> *>(*dst);
     if (mode == 1) {
-        t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, no_kappa) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, no_kappa);
-        tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, no_kappa);
+        t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, no_kappa) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, no_kappa, roots);
+        tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, no_kappa, roots);
     } else {
         t = tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, 0);
         if (mode == 2) {
-            t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK) : tau_gen(t, nA, TAU_LEVELS, 0, lgK);
-            tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK);
+            t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, false, roots);
+            tau_gen(t, k.lgB, TAU_POWERS, lgL, lgK, false, roots);
         }
     }
     PACO_CUDA_TRY(cudaGetLastError());
@@ -191,10 +228,7 @@ static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerK
     a->lo_bits = pl->twN_lo_bits;
     a->n_mask = (unsigned)(pl->N - 1);
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    void *w = nullptr;
-    paco_status_t st = gen_table(8, &w, 1LL << lgL, 1LL << lgL, 1, 0);
-    if (st == PACO_OK) st = power_table(static_cast<const cx<float> *>(w), lgL, tw);
-    cudaFree(w);
+    const paco_status_t st = power_table(static_cast<const cx<float> *>(i == 0 ? pl->twL1 : pl->twL2), lgL, tw);
     a->twL = static_cast<const cx<float> *>(*tw);
     return st;
 }

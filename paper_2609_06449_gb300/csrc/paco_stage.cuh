@@ -67,21 +67,6 @@ __device__ __forceinline__ cx<double> ldg_cx<double>(const cx<double> *p)
 }
 
 template <typename R>
-__device__ __forceinline__ cx<R> ldcg_cx(const cx<R> *p);
-template <>
-__device__ __forceinline__ cx<float> ldcg_cx<float>(const cx<float> *p)
-{
-    float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
-    return make_cx<float>(v.x, v.y);
-}
-template <>
-__device__ __forceinline__ cx<double> ldcg_cx<double>(const cx<double> *p)
-{
-    double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
-    return make_cx<double>(v.x, v.y);
-}
-
-template <typename R>
 __device__ __forceinline__ void st_cx(cx<R> *p, cx<R> v) { *p = v; }
 
 // Dynamic shared memory needed by a stage CTA (elements of cx<R>).
@@ -104,8 +89,6 @@ __host__ __device__ inline int stage_smem_elems(int A, int B, int K, int W, int 
 //
 // stage_tile is the body: one tile (`tile`, transform base offset `boff`,
 // cluster rank `rank`) computed by the calling CTA's NT = NE / EPT threads.
-// LDCG loads the tile input through L2 only (ld.global.cg): for inputs that
-// other CTAs of the same launch wrote (the batched persistent kernel).
 // FORM != TC_NONE computes the radix-16 passes (F1 and F2 pass 1 when the
 // radix is 16) as tensor-core contractions (paco_tc.cuh); its fragment table
 // and per-warp staging follow the stage's shared memory.
@@ -115,7 +98,7 @@ __host__ __device__ inline int stage_smem_elems(int A, int B, int K, int W, int 
 // sharded form's addresses (ShardArgs): Phase I on a local input slab with
 // global twiddle columns, stored into the G send blocks; Phase III reading
 // the received blocks; the output offset of the transform is boff_out.
-template <typename R, int A, int B, int LGWC, int LGKC, int MC, bool LDCG, int FORM = TC_NONE, int TERMS = 0,
+template <typename R, int A, int B, int LGWC, int LGKC, int MC, int FORM = TC_NONE, int TERMS = 0,
           bool SHARD = false, int SPLIT = 0>
 __device__ __forceinline__ void stage_tile(const StageArgs &args, int tile, long long boff, int rank,
                                            unsigned char *smem_raw, const StageTerms *terms = nullptr,
@@ -283,8 +266,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &args, int tile, long
                     if (sp->sub != 3) row = (unsigned)j;               // natural rows (sub 3: pi over La's digits)
                     x = ldg_cx(gin + (long long)row * args.C + cbase + col);
                 } else {
-                    x = LDCG ? ldcg_cx(gin + (long long)row * args.C + c0 + col)
-                             : ldg_cx(gin + (long long)row * args.C + c0 + col);
+                    x = ldg_cx(gin + (long long)row * args.C + c0 + col);
                 }
                 if constexpr (TERMS == 1) if (ldw) {
                     R f = lds;
@@ -580,7 +562,7 @@ __global__ void __launch_bounds__(512, MINB) paco_stage_kernel(const StageArgs a
     const int lgK = (LGKC >= 0) ? LGKC : args.lgK;
     int rank = 0;
     if ((1 << lgK) > 1) rank = (int)cg::this_cluster().block_rank();
-    stage_tile<R, A, B, LGWC, LGKC, MC, false, FORM>(args, (int)(blockIdx.x >> lgK),
+    stage_tile<R, A, B, LGWC, LGKC, MC, FORM>(args, (int)(blockIdx.x >> lgK),
                                                      (long long)blockIdx.y * args.batch_stride, rank, smem_raw);
 }
 
@@ -593,7 +575,7 @@ __global__ void __launch_bounds__(512, MINB) paco_stage_kernel_shard(const Stage
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int rank = 0;
     if ((1 << args.lgK) > 1) rank = (int)cg::this_cluster().block_rank();
-    stage_tile<R, A, B, -1, -1, 0, false, TC_NONE, 0, true>(
+    stage_tile<R, A, B, -1, -1, 0, TC_NONE, 0, true>(
         args, (int)(blockIdx.x >> args.lgK), (long long)blockIdx.y * in_stride, rank, smem_raw, nullptr, &sh,
         (long long)blockIdx.y * out_stride);
 }
@@ -603,7 +585,7 @@ template <typename R, int A, int B, int MINB>
 __global__ void __launch_bounds__(512, MINB) paco_stage_kernel_split(const StageArgs args, const SplitArgs sp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    stage_tile<R, A, B, -1, 0, 0, false, TC_NONE, 0, false, 1>(
+    stage_tile<R, A, B, -1, 0, 0, TC_NONE, 0, false, 1>(
         args, (int)blockIdx.x, (long long)blockIdx.y * args.batch_stride, 0, smem_raw, nullptr, nullptr, 0, &sp);
 }
 
@@ -616,7 +598,7 @@ __global__ void __launch_bounds__(512, MINB) paco_stage_kernel_terms(const Stage
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int rank = 0;
     if ((1 << args.lgK) > 1) rank = (int)cg::this_cluster().block_rank();
-    stage_tile<R, A, B, -1, -1, 0, false, TC_NONE, TM>(args, (int)(blockIdx.x >> args.lgK),
+    stage_tile<R, A, B, -1, -1, 0, TC_NONE, TM>(args, (int)(blockIdx.x >> args.lgK),
                                                          (long long)blockIdx.y * args.batch_stride, rank, smem_raw,
                                                          &terms);
 }
