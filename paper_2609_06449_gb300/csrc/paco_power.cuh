@@ -9,9 +9,9 @@
 // bit permutations (pi in any base 2^t is one), so the row of j is the sum of a
 // per-thread term for j_lo and one of at most 32 launch constants for j_hi.
 //
-// Measured on GB300, 256 x 2^20: Phase I 1.39 -> 1.0 ms, Phase III with the sum
-// 1.92 -> 0.95 ms against the generic stage kernels, which spend 130-140 warp
-// instructions a point on run-time strides and twiddle products.
+// Measured on GB300, 256 x 2^20 with the sum: 3.34 -> 1.86 ms against the generic
+// stage kernels, which spend 130-140 warp instructions a point on run-time
+// strides and twiddle products.
 #pragma once
 
 #include "../../include/paco.h"
