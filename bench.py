@@ -274,26 +274,32 @@ def workload_config(args):
     }
 
 
-def captured_traffic(N1: int, N2: int, b: int, p: int, dtype: str, dir: int):
-    """DRAM bytes per launch (mean of the passes) from the committed ncu capture
-    (profiles/roofline_traffic.json), or None when the workload differs or the
-    kernel source changed since the counters were taken."""
+def captured_traffic(stage: str, N1: int, N2: int, b: int, p: int, dtype: str, dir: int):
+    """DRAM bytes per launch from the committed ncu captures
+    (profiles/roofline_traffic.json): "stage1" / "stage2" of the panel kernel,
+    "passes" the mean pass of paco_execute.  None when the workload differs or
+    the kernel source changed since the counters were taken."""
     import hashlib
     if (N1, N2, b, p, dtype, dir) != (1 << 14, 1 << 14, 4, 64, "c64", -1):
         return None
     try:
         with open(os.path.join(ROOT, "profiles", "roofline_traffic.json")) as fh:
             rec = json.load(fh)
+        if stage == "passes":
+            rec, names = rec["passes"], ("paco_fold.cuh", "paco_common.cuh")
+        else:
+            names = ("paco_panel.cuh", "paco_common.cuh")
         csrc = os.path.join(ROOT, "paper_2609_06449_gb300", "csrc")
         h = hashlib.sha256()
-        for name in ("paco_fold.cuh", "paco_common.cuh"):
+        for name in names:
             with open(os.path.join(csrc, name), "rb") as fh:
                 h.update(fh.read())
         if h.hexdigest()[:16] != rec["source_sha16"]:
             return None
-        per = rec["traffic_bytes_per_launch"]
-        return float(sum(per) / len(per))
-    except (OSError, KeyError, TypeError, ValueError):
+        if stage == "passes":
+            return float(sum(rec["bytes_per_launch"]) / len(rec["bytes_per_launch"]))
+        return float(rec["traffic_bytes_per_launch"][stage])
+    except (OSError, KeyError, ValueError):
         return None
 
 
@@ -936,7 +942,7 @@ def main():
     hbm_eff = 4.0 * N * esize * world / (ms_step * 1e-3) / 1e9
 
     pass_ms = total_ms / K / launches             # mean launch
-    traffic = captured_traffic(N1, N2, args.b, args.p, args.dtype, args.dir)
+    traffic = captured_traffic("passes", N1, N2, args.b, args.p, args.dtype, args.dir)
     bytes_per_launch = 2.0 * N * esize            # read N + write N elements
     achieved = bytes_per_launch / (pass_ms * 1e-3) / 1e9
     peak, peak_src = measured_peak_hbm()
