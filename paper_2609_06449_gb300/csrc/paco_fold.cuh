@@ -13,7 +13,7 @@
 // butterflies.  In complex128, which the FP64 pipe bounds, the count is the
 // time (2^27: 109 operations a point and 27.5 ms with separate products in the
 // stage kernels).  In complex64 it is the issue rate: a pass of 1024 points
-// over 2^28 went from 1.38 ms (139 instructions a point) to 0.76-0.93 ms.
+// over 2^28 went from 1.38 ms (139 instructions a point) to 0.76-0.85 ms.
 //
 // A pass transforms L = A B rows (j = j_hi B + j_lo, k = k_lo + A k_hi) of a
 // tile of W columns: A-point DFTs over j_hi in registers, one exchange through
@@ -33,8 +33,9 @@
 // factors shows: with all factors as products of rounded values the relative
 // error of 2^24 points is 2.2e-7, with the tables above 1.9e-7 (the stage
 // kernels: 2.0e-7).  2 E - p carries p's rounding on; in FP64, whose error is
-// held to the stage kernels' too, TW 1 therefore multiplies F1's rows first
-// and takes the plain DFT (ROWS).
+// held to the stage kernels' too, F1 therefore multiplies its rows first and
+// takes the plain DFT (ROWS; 2^27: 21.1 ms, 19.6 with F1 folded at an error 1 to
+// 7 % larger).
 #pragma once
 
 #include "../../include/paco.h"
@@ -196,7 +197,7 @@ struct FoldCfg {
     static constexpr int EPT = EPT_ ? EPT_ : A > B ? (A > 16 ? A : 16) : (B > 16 ? B : 16);
     static constexpr int NT = L * W / EPT;
     static constexpr int U1 = EPT / A, U2 = EPT / B;
-    // exchange layouts as in paco_pass.cuh; PH points make one shared-memory phase
+    // exchange layouts as in paco_power.cuh; PH points make one shared-memory phase
     static constexpr int PH = sizeof(R) == 4 ? 16 : 8;
     static constexpr int SJ = FIRST ? A + 1 : W;
     static constexpr int SC0 = B * SJ;
