@@ -228,6 +228,36 @@ struct FoldCfg {
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A load of the caller's data (transform, weights, scale) in such a kernel: the
+// kernel before may still be writing it when this one starts, so it is neither
+// __ldg (the read-only path asks for data that nothing writes as long as the
+// kernel runs, its wait included) nor a load that the compiler may move over
+// grid_wait (volatile).  Through L2, as the passes run in place.
+__device__ __forceinline__ float ld_data(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_data(const double *p)
+{
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_data(const float2 *p)
+{
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_data(const double2 *p)
+{
+    double2 v;
+    asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
 // One tile of the transform at element offset boff (PDL: the tile's kernel was
 // launched with programmatic serialisation).
 template <class CFG, bool PDL = false>
@@ -283,13 +313,13 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
         if (a.conj) {
 #pragma unroll
             for (int r = 0; r < A; ++r) {
-                const V t = __ldcg(p + a.rowA[r]);
+                const V t = ld_data(p + a.rowA[r]);
                 v[u * A + r] = make_cx<R>(t.y, t.x);
             }
         } else {
 #pragma unroll
             for (int r = 0; r < A; ++r) {
-                const V t = __ldcg(p + a.rowA[r]);
+                const V t = ld_data(p + a.rowA[r]);
                 v[u * A + r] = make_cx<R>(t.x, t.y);
             }
         }
@@ -366,7 +396,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             const unsigned c = c0 + col;
             const unsigned row = a.crev_bits ? digit_reverse(c, a.crev_bits, a.crev_t) : c;
             q = reinterpret_cast<V *>(a.out + boff + (long long)row * a.ld_out + klo);
-            const R f = a.scale ? a.mult * (R)__ldg(a.scale) : a.mult;
+            const R f = a.scale ? a.mult * (R)ld_data(a.scale) : a.mult;
             if (f != R(1)) {
 #pragma unroll
                 for (int k = 0; k < B; ++k) v[u * B + k] = make_cx<R>(v[u * B + k].x * f, v[u * B + k].y * f);

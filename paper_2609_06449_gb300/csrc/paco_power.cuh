@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_power_kernel(const __
         const float2 *p = reinterpret_cast<const float2 *>(a.in + base + col + (long long)jrow * a.ld_in);
 #pragma unroll
         for (int r = 0; r < A; ++r) {
-            const float2 t = __ldcg(p + a.rowA[r]);
+            const float2 t = ld_data(p + a.rowA[r]);
             v[u * A + r] = make_cx<float>(t.x, t.y * sg);
         }
     }
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_power_kernel(const __
                 float wv[H];
 #pragma unroll
                 for (int i = 0; i < H; ++i)
-                    wv[i] = __ldg(a.w + o + a.rowK[B == 32 ? g + 2 * (i >> 1) + 16 * (i & 1) : i]);
+                    wv[i] = ld_data(a.w + o + a.rowK[B == 32 ? g + 2 * (i >> 1) + 16 * (i & 1) : i]);
                 float &pw = power[B == 32 ? g : NP == 1 ? 0 : u];
 #pragma unroll
                 for (int i = 0; i < H; ++i) {

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::CTAS) paco_tcpass_kernel(const _
         const float2 *p = reinterpret_cast<const float2 *>(a.in + base + col + (long long)jrow * a.ld_in) + rq;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const float2 t = __ldcg(p + ((i & 1) ? a.rowA[1] : 0u) + ((i & 2) ? a.rowA[8] : 0u));
+            const float2 t = ld_data(p + ((i & 1) ? a.rowA[1] : 0u) + ((i & 2) ? a.rowA[8] : 0u));
             x[nt][i] = a.conj ? make_cx<float>(t.y, t.x) : make_cx<float>(t.x, t.y);
         }
     }
