@@ -304,6 +304,8 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
     }
     if constexpr (PDL) grid_wait();
     // ---- F1
+    [[maybe_unused]] R f = R(1);
+    if constexpr (FIRST) f = a.scale ? a.mult * (R)ld_data(a.scale) : a.mult;
     C v[CFG::EPT];
 #pragma unroll
     for (int u = 0; u < U1; ++u) {
@@ -322,6 +324,13 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
                 const V t = ld_data(p + a.rowA[r]);
                 v[u * A + r] = make_cx<R>(t.x, t.y);
             }
+        }
+    }
+    if constexpr (FIRST) {
+        // the input, not the result: a sum may overflow where the scaled one does not
+        if (f != R(1)) {
+#pragma unroll
+            for (int i = 0; i < CFG::EPT; ++i) v[i] = make_cx<R>(v[i].x * f, v[i].y * f);
         }
     }
     if constexpr (TW == 2) {
@@ -396,11 +405,6 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             const unsigned c = c0 + col;
             const unsigned row = a.crev_bits ? digit_reverse(c, a.crev_bits, a.crev_t) : c;
             q = reinterpret_cast<V *>(a.out + boff + (long long)row * a.ld_out + klo);
-            const R f = a.scale ? a.mult * (R)ld_data(a.scale) : a.mult;
-            if (f != R(1)) {
-#pragma unroll
-                for (int k = 0; k < B; ++k) v[u * B + k] = make_cx<R>(v[u * B + k].x * f, v[u * B + k].y * f);
-            }
         } else {
             q = reinterpret_cast<V *>(a.out + base + col + (long long)klo * a.ld_out);
         }

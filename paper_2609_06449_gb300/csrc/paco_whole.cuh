@@ -53,7 +53,7 @@ struct WholeCfg {
 };
 
 // Step I of the tile's transforms.  off(g): element offset of transform g, or
-// negative where the tile has none; f multiplies the result.
+// negative where the tile has none; f multiplies the input.
 template <class CFG, int EPT, int NT, int I, class Off>
 __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
                                            const Off &off, cx<float> *sm)
@@ -91,6 +91,10 @@ __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool c
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u * R + r] = make_cx<float>(v[u * R + r].y, v[u * R + r].x);
             }
+            if (f != 1.f) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[u * R + r] = make_cx<float>(v[u * R + r].x * f, v[u * R + r].y * f);
+            }
             plain_dft<R>(v + u * R);
         } else {
             // (up to 2^7 points the copy rate leaves room for the closer form)
@@ -107,10 +111,6 @@ __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool c
             const long long o = off(g);
             if (o >= 0) {
                 float2 *q = out + o + kap;
-                if (f != 1.f) {
-#pragma unroll
-                    for (int k = 0; k < R; ++k) v[u * R + k] = make_cx<float>(v[u * R + k].x * f, v[u * R + k].y * f);
-                }
                 if (conj) {
 #pragma unroll
                     for (int k = 0; k < R; ++k) q[K * k] = make_float2(v[u * R + k].y, v[u * R + k].x);

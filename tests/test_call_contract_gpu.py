@@ -1,9 +1,13 @@
 """What a call owes its caller whichever kernels run it: data written by the
-kernel just before it in the stream is what it reads."""
+kernel just before it in the stream is what it reads, and the scalar of a
+weighted input multiplies the input."""
+
+import math
 
 import numpy as np
 import pytest
 
+import oracle
 from paco_inputs import gaussian, weights
 
 torch = pytest.importorskip("torch")
@@ -44,3 +48,23 @@ def test_weights_and_scale_written_just_before_the_call(l1, l2, batch):
     plan.check()
     for k in range(20):
         assert torch.equal(got[k], want[k]), k
+
+
+@pytest.mark.parametrize("size,mult,scale", [(1e37, 1e-10, None), (1e37, 0.5, 1e-9), (1e-41, 1e12, None), (1e-41, 4.0, 1e11)])
+@pytest.mark.parametrize("l1,l2,batch", [(2, 2, 9), (3, 3, 5), (4, 4, 3), (6, 6, 3), (7, 6, 33), (7, 7, 2), (8, 8, 3), (9, 9, 2), (10, 10, 1),
+                                         (11, 11, 1)])
+def test_the_scalar_multiplies_the_input(l1, l2, batch, size, mult, scale):
+    """Inputs whose sums overflow, or that are subnormal, before they are scaled
+    and neither afterwards; bound of the complex64 transform."""
+    N = 1 << (l1 + l2)
+    x = (gaussian(batch * N, l1 + 5 * l2, np.complex64) * np.float32(size)).astype(np.complex64).reshape(batch, N)
+    plan = paco.Plan(1 << l1, 1 << l2, 2, batch, paco.C64)
+    xt = torch.from_numpy(x).cuda()
+    y = torch.empty_like(xt)
+    st = None if scale is None else torch.tensor(scale, dtype=torch.float64, device="cuda")
+    plan.execute_weighted_input(xt, y, None, st, mult, -1)
+    torch.cuda.synchronize()
+    f = np.float32(mult) * np.float32(1.0 if scale is None else scale)
+    ref = oracle.fft(x.astype(np.complex128) * float(f), threads=0)
+    err = np.linalg.norm(y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert np.max(err) <= 5e-7 * math.log2(N)
