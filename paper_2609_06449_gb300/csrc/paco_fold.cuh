@@ -60,7 +60,7 @@ struct FoldArgs {
     int lg_n, lg_k;         // log2 N, log2 K
     int conj;               // 1: the conjugate transform
     int reverse;            // 1: tiles from the last to the first
-    R mult;                 // FIRST: the input is scaled by mult * (*scale or 1)
+    R mult;                 // SCALED: the input is scaled by mult * (*scale or 1)
     const double *scale;
 };
 
@@ -187,11 +187,13 @@ __device__ __forceinline__ void fold_dft(cx<R> *v, const Tau &tau)
 __host__ __device__ constexpr bool fold_plain(bool fp64, int lgB) { return fp64 || lgB < 4; }
 
 // EPT_: points a thread holds (0: 16, or 32 where a factor needs them).
-template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0>
+// SCALED_: FIRST with FoldArgs::mult and scale (a kernel of its own: with a branch in
+// the one kernel 23 x 1024^2 went from 145 to 147 us).
+template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0, bool SCALED_ = false>
 struct FoldCfg {
     using R = R_;
     static constexpr int LGA = LGA_, LGB = LGB_, LGW = LGW_;
-    static constexpr bool FIRST = FIRST_;
+    static constexpr bool FIRST = FIRST_, SCALED = SCALED_;
     static constexpr int TW = FIRST_ ? 0 : TW_;
     static constexpr int A = 1 << LGA, B = 1 << LGB, W = 1 << LGW, L = A * B;
     static constexpr int EPT = EPT_ ? EPT_ : A > B ? (A > 16 ? A : 16) : (B > 16 ? B : 16);
@@ -305,7 +307,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
     if constexpr (PDL) grid_wait();
     // ---- F1
     [[maybe_unused]] R f = R(1);
-    if constexpr (FIRST) f = a.scale ? a.mult * (R)ld_data(a.scale) : a.mult;
+    if constexpr (CFG::SCALED) f = a.scale ? a.mult * (R)ld_data(a.scale) : a.mult;
     C v[CFG::EPT];
 #pragma unroll
     for (int u = 0; u < U1; ++u) {
@@ -326,12 +328,10 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             }
         }
     }
-    if constexpr (FIRST) {
+    if constexpr (CFG::SCALED) {
         // the input, not the result: a sum may overflow where the scaled one does not
-        if (f != R(1)) {
 #pragma unroll
-            for (int i = 0; i < CFG::EPT; ++i) v[i] = make_cx<R>(v[i].x * f, v[i].y * f);
-        }
+        for (int i = 0; i < CFG::EPT; ++i) v[i] = make_cx<R>(v[i].x * f, v[i].y * f);
     }
     if constexpr (TW == 2) {
         if constexpr (CFG::EPT != 32) load_twiddles();
@@ -408,12 +408,22 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
         } else {
             q = reinterpret_cast<V *>(a.out + base + col + (long long)klo * a.ld_out);
         }
+        // parts swapped back: at the stores, or (first pass of 512 points) in a branch
+        // before them, which keeps the stores behind all of the sequence's F2 (200 x
+        // 2^18: 261 us, with selects 273; 301 x 2^16, with a first pass of 256: 97 and 95)
+        constexpr bool SWAP = FIRST && CFG::EPT == 32 && U2 > 1;
+        if constexpr (SWAP) {
+            if (a.conj) {
+#pragma unroll
+                for (int k = 0; k < B; ++k) v[u * B + k] = make_cx<R>(v[u * B + k].y, v[u * B + k].x);
+            }
+        }
 #pragma unroll
         for (int k = 0; k < B; ++k) {
             const C y = v[u * B + k];
             V o;
-            o.x = a.conj ? y.y : y.x;
-            o.y = a.conj ? y.x : y.y;
+            o.x = !SWAP && a.conj ? y.y : y.x;
+            o.y = !SWAP && a.conj ? y.x : y.y;
             if constexpr (FIRST) q[A * k] = o;
             else __stcs(q + a.rowK[k], o);
         }
@@ -461,8 +471,9 @@ template <typename R>
 paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa = false);
 
 // The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
-// (the row stride); fn == nullptr where none is built.
-FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC, bool narrow);
+// (the row stride); fn == nullptr where none is built.  scaled: the first pass of a
+// scaled input.
+FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC, bool narrow, bool scaled = false);
 FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC);
 
 } // namespace paco

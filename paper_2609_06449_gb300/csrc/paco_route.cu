@@ -31,6 +31,7 @@ struct Route {
     int n = 0;                     // passes of paco_execute (0: the stage kernels)
     WholeKernel whole;             // n = 1: whole transforms in a CTA
     FoldKernel k[MAX_PASSES];
+    FoldKernel scaled;                 // k[0] for a scaled input (complex64)
     int twmode[MAX_PASSES] = {};       // FoldCfg::TW
     FoldArgs<float> f[MAX_PASSES];     // by the plan's precision
     FoldArgs<double> d[MAX_PASSES];
@@ -312,7 +313,11 @@ paco_status_t route_setup(paco_plan *pl)
         r->k[i] = pl->esize == 8 ? fold_kernel_f32(i == 0, r->twmode[i], f[i], lgC, pl->N * pl->batch <= (int64_t)1 << 24)
                                  : fold_kernel_f64(i == 0, r->twmode[i], f[i], lgC);
         if (!r->k[i].fn) n = 0;
+        if (i == 0 && pl->esize == 8)
+            r->scaled = fold_kernel_f32(true, 0, f[i], lgC, pl->N * pl->batch <= (int64_t)1 << 24, true);
     }
+    if (n && r->scaled.fn)
+        PACO_CUDA_TRY(cudaFuncSetAttribute(r->scaled.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->scaled.smem));
     // pi of the redistribution: the plan's base where its digits fit the factors
     int t = pl->t;
     for (int i = 1; i < n; ++i)
@@ -365,11 +370,13 @@ static paco_status_t run_passes(const paco_plan *pl, const FoldArgs<R> *args, co
         a.out = static_cast<cx<R> *>(out);
         a.conj = dir == 1;
         a.reverse = i & 1;
-        if (terms && i == 0) {
+        const bool scaled = terms && i == 0;
+        if (scaled) {
             a.mult = (R)terms->ld_mult;
             a.scale = terms->ld_scale;
         }
-        const paco_status_t st = launch(pl, r.k[i].fn, &a, (long long)pl->batch << a.lg_all, r.k[i].threads, r.k[i].smem, true, stream);
+        const FoldKernel &k = scaled ? r.scaled : r.k[i];
+        const paco_status_t st = launch(pl, k.fn, &a, (long long)pl->batch << a.lg_all, k.threads, k.smem, true, stream);
         if (st != PACO_OK) return st;
     }
     return PACO_OK;
