@@ -100,24 +100,30 @@ template <int LG, bool FIRST>
 using StageCfgB = FoldCfg<float, LG == 9 || LG == 10 ? 5 : LG == 6 ? 3 : 4, LG == 10 ? 5 : LG >= 8 ? 4 : 3, 13 - LG, FIRST,
                           1, batched::EPT>;
 
-template <bool FIRST>
-__device__ __forceinline__ void stage_item(const FoldArgs<float> &sa, int lgL, int tile, long long boff, unsigned char *smem)
+template <bool FIRST, bool AGAIN = false>
+__device__ __forceinline__ bool stage_item(const FoldArgs<float> &sa, int lgL, int tile, long long boff, unsigned char *smem)
 {
     switch (lgL) {
-    case 6: fold_tile<StageCfgB<6, FIRST>>(sa, tile, boff, smem); break;
-    case 7: fold_tile<StageCfgB<7, FIRST>>(sa, tile, boff, smem); break;
-    case 8: fold_tile<StageCfgB<8, FIRST>>(sa, tile, boff, smem); break;
-    case 9: fold_tile<StageCfgB<9, FIRST>>(sa, tile, boff, smem); break;
-    case 10: fold_tile<StageCfgB<10, FIRST>>(sa, tile, boff, smem); break;
-    default: break;
+    case 6: return fold_tile<StageCfgB<6, FIRST>, false, AGAIN>(sa, tile, boff, smem);
+    case 7: return fold_tile<StageCfgB<7, FIRST>, false, AGAIN>(sa, tile, boff, smem);
+    case 8: return fold_tile<StageCfgB<8, FIRST>, false, AGAIN>(sa, tile, boff, smem);
+    case 9: return fold_tile<StageCfgB<9, FIRST>, false, AGAIN>(sa, tile, boff, smem);
+    case 10: return fold_tile<StageCfgB<10, FIRST>, false, AGAIN>(sa, tile, boff, smem);
+    default: return false;
     }
+}
+
+// (out of line: it takes no register of the common path)
+__device__ __noinline__ void stage_again(const FoldArgs<float> &sa, int lgL, int tile, long long boff, unsigned char *smem)
+{
+    stage_item<false, true>(sa, lgL, tile, boff, smem);
 }
 
 template <int LG>
 __device__ __forceinline__ void small_item(const BatchedArgs &a, const float2 *tau, int count, const long long *s_off,
                                            unsigned char *smem)
 {
-    whole_step<WholeCfg<LG, batched::EPT, batched::NT>, batched::EPT, batched::NT, 0>(
+    whole_tile<WholeCfg<LG, batched::EPT, batched::NT>, batched::EPT, batched::NT>(
         static_cast<const float2 *>(a.in), static_cast<float2 *>(a.out), a.conj != 0, 1.f, tau,
         [&](int g) { return g < count ? s_off[g] : -1ll; }, reinterpret_cast<cx<float> *>(smem));
 }
@@ -213,7 +219,8 @@ __global__ void __launch_bounds__(batched::NT, 2) paco_batched_kernel(const __gr
             }
             __syncthreads();
             if (!s_ok) continue;                  // reported through the status word
-            stage_item<false>(s_sa, ld.lg2, item.b, item.off, smem_raw);
+            if (stage_item<false>(s_sa, ld.lg2, item.b, item.off, smem_raw))
+                stage_again(s_sa, ld.lg2, item.b, item.off, smem_raw);
         } else {
             __syncthreads();                      // s_sa written
             stage_item<true>(s_sa, ld.lg1, item.b, item.off, smem_raw);

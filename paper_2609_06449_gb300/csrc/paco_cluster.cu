@@ -118,7 +118,7 @@ __device__ __forceinline__ void dft256_finish(cx<float> *v, float2 *buf, int W, 
     const int col2 = T16_FAST ? tid / 16 : tid % W, u = T16_FAST ? tid % 16 : tid / W;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = ld_cx(&buf[(u * 16 + t) * W + (col2 ^ u)]);
-    fold_dft<true, float, 16>(v, [&](int q) { return make_cx<float>(f[q].x, f[q].y); });
+    fold_dft<DIRECT, float, 16>(v, [&](int q) { return make_cx<float>(f[q].x, f[q].y); });
 }
 
 } // namespace
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(4096 / K, K == 16 ? 2 : 1) paco_cluster_kernel
         const int j = u16 + 16 * s;
         v[s] = ld_cx(&bufB[j * W2 + vl]);                     // row j mod W1 of the block from CTA j / W1
     }
-    fold_dft<true, float, 16>(v, [&](int i) { return make_cx<float>(f3a[i].x, f3a[i].y); });
+    fold_dft<DIRECT, float, 16>(v, [&](int i) { return make_cx<float>(f3a[i].x, f3a[i].y); });
     dft256_finish<false>(v, bufA, W2, vl, u16, f3b);          // (every read of bufA was before the exchange)
 #pragma unroll
     for (int k = 0; k < 16; ++k) {

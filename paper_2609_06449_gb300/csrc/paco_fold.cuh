@@ -71,13 +71,27 @@ template <> struct vec2<double> { using type = double2; };
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// (e, o) -> (e + t o, e - t o), the second as 2 e - (e + t o) or (DIRECT) on its
-// own: two more operations, and p's rounding is not carried on.
-template <bool DIRECT, typename R>
+// (e, o) -> (e + t o, e - t o).
+// CARRY: the second as 2 e - (e + t o).
+// DIRECT: on its own, two more operations; the first one's rounding is not carried on.
+// SAFE: where a sum may overflow.  CARRY then takes the finite difference beside
+// an overflowing sum with it, and a product with a zero part of t makes a NaN of
+// an infinite o: here each part overflows on its own.
+enum Bfly { CARRY, DIRECT, SAFE };
+template <int KIND, typename R>
 __device__ __forceinline__ void bfly(cx<R> &e, cx<R> &o, cx<R> t)
 {
+    if constexpr (KIND == SAFE) {
+        cx<R> m;
+        if (t.y == R(0)) m = make_cx<R>(t.x * o.x, t.x * o.y);
+        else if (t.x == R(0)) m = make_cx<R>(-t.y * o.y, t.y * o.x);
+        else m = make_cx<R>(fma_r(t.x, o.x, -(t.y * o.y)), fma_r(t.x, o.y, t.y * o.x));
+        o = make_cx<R>(e.x - m.x, e.y - m.y);
+        e = make_cx<R>(e.x + m.x, e.y + m.y);
+        return;
+    }
     const R px = fma_r(-t.y, o.y, fma_r(t.x, o.x, e.x)), py = fma_r(t.y, o.x, fma_r(t.x, o.y, e.y));
-    if constexpr (DIRECT)
+    if constexpr (KIND == DIRECT)
         o = make_cx<R>(fma_r(t.y, o.y, fma_r(-t.x, o.x, e.x)), fma_r(-t.y, o.x, fma_r(-t.x, o.y, e.y)));
     else
         o = make_cx<R>(fma_r(R(2), e.x, -px), fma_r(R(2), e.y, -py));
@@ -145,7 +159,7 @@ __device__ __forceinline__ void plain_dft(cx<R> *v)
 // tau(q) with q = tau_index(n, s) is T^(RADIX / n) w_n^{-s}, s < n / 4 (s = 0 for n = 2, 4).
 __host__ __device__ constexpr int tau_index(int n, int s) { return n == 2 ? 0 : n / 4 + s; }
 
-template <bool DIRECT, typename R, int RADIX, int N_, class Tau>
+template <int KIND, typename R, int RADIX, int N_, class Tau>
 __device__ __forceinline__ void fold_level(cx<R> *u, const Tau &tau)
 {
     constexpr int Q = N_ >= 4 ? N_ / 4 : 1;
@@ -154,11 +168,11 @@ __device__ __forceinline__ void fold_level(cx<R> *u, const Tau &tau)
         const cx<R> t = tau(tau_index(N_, s));
 #pragma unroll
         for (int b = 0; b < RADIX; b += N_) {
-            bfly<DIRECT>(u[b + s], u[b + s + N_ / 2], t);
-            if constexpr (N_ >= 4) bfly<DIRECT>(u[b + s + Q], u[b + s + Q + N_ / 2], make_cx<R>(t.y, -t.x));
+            bfly<KIND>(u[b + s], u[b + s + N_ / 2], t);
+            if constexpr (N_ >= 4) bfly<KIND>(u[b + s + Q], u[b + s + Q + N_ / 2], make_cx<R>(t.y, -t.x));
         }
     }
-    if constexpr (N_ < RADIX) fold_level<DIRECT, R, RADIX, N_ * 2>(u, tau);
+    if constexpr (N_ < RADIX) fold_level<KIND, R, RADIX, N_ * 2>(u, tau);
 }
 
 template <int RADIX>
@@ -170,15 +184,38 @@ __host__ __device__ constexpr int bitrev_c(int i)
 }
 
 // v[k] = sum_r v[r] T^r w_RADIX^{-rk}
-template <bool DIRECT, typename R, int RADIX, class Tau>
+template <int KIND, typename R, int RADIX, class Tau>
 __device__ __forceinline__ void fold_dft(cx<R> *v, const Tau &tau)
 {
     cx<R> u[RADIX];
 #pragma unroll
     for (int i = 0; i < RADIX; ++i) u[i] = v[bitrev_c<RADIX>(i)];
-    fold_level<DIRECT, R, RADIX, 2>(u, tau);
+    fold_level<KIND, R, RADIX, 2>(u, tau);
 #pragma unroll
     for (int i = 0; i < RADIX; ++i) v[i] = u[i];
+}
+
+// Whether one of N values is so large that a sum of 2^lg of them (a DFT's result, or
+// a partial one: at most sqrt(2) 2^lg times the largest part) may overflow.  Every
+// tile of CARRY butterflies asks this of its input at its exchange's barrier, and
+// is done again with SAFE ones where one thread says yes.
+template <int N>
+__device__ __forceinline__ bool may_overflow(const cx<float> *v, int lg)
+{
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(m), "f"(v[i].x), "f"(v[i].y));
+    return m >= __uint_as_float((unsigned)(127 + 126 - lg) << 23);
+}
+template <int N>
+__device__ __forceinline__ bool may_overflow(const cx<double> *v, int lg)
+{
+    // by the high words: the FP64 pipe is what bounds these passes
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        m = max(max(m, __double2hiint(v[i].x) & 0x7fffffff), __double2hiint(v[i].y) & 0x7fffffff);
+    return m >= (1023 + 1022 - lg) << 20;
 }
 
 // With kappa = 0, F2 is plain and w_L^{-k_lo j_lo} a product of its own in FP64 and
@@ -212,9 +249,15 @@ struct FoldCfg {
     // 0.648 -> 0.610 ms).  With 32 they cost more than they hide: 512 0.66 -> 0.72;
     // 1024 0.853 -> 0.834, but one 2^20 12.3 -> 14.3 us.
     static constexpr bool AHEAD = TW == 1 && !FP64 && EPT == 16;
-    // F2's butterflies in the closer form (bfly), but where the error has room
-    static constexpr bool DIRECT = TW != 1 && !FP64 && (FIRST || TW == 2 || LGB < 5);
     static constexpr bool ROWS = TW && FP64;                      // F1's factors by row (T^r), not by level
+    // The butterflies of F1 and F2 (bfly): CARRY with may_overflow's question, or DIRECT
+    // where that costs less.  us without the question, with it, and with DIRECT: 16 x
+    // 2^24 (256 points) 2012, 2013, 2073; 50 x 2^20 (1024 points, TW 1) 326.8, 327.4,
+    // 337.9; but 2^28 (512 points, TW 2) 2283, 2385, 2345, and the 2-D form's 1024 points
+    // (23 x 1024^2) 144.8, 150.8, 146.4.
+    static constexpr int BFLY1 = TW == 2 && EPT == 32 ? DIRECT : CARRY;
+    static constexpr int BFLY2 = TW != 1 && !FP64 ? DIRECT : CARRY;
+    static constexpr bool CARRIES = (TW && !ROWS && BFLY1 == CARRY) || (!PLAIN2 && BFLY2 == CARRY);
     static constexpr int NA = ROWS ? A : A / 2;                   // factors of F1, a column
     static constexpr int NTW = TW == 2 ? (NA + LGB) * W : 0;
     static constexpr int SMEM = (EX + NTW) * 2 * (int)sizeof(R);
@@ -261,9 +304,10 @@ __device__ __forceinline__ double2 ld_data(const double2 *p)
 }
 
 // One tile of the transform at element offset boff (PDL: the tile's kernel was
-// launched with programmatic serialisation).
-template <class CFG, bool PDL = false>
-__device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, int tile, long long boff,
+// launched with programmatic serialisation).  True: nothing was stored, the tile
+// is to be done with AGAIN (may_overflow).
+template <class CFG, bool PDL = false, bool AGAIN = false>
+__device__ __forceinline__ bool fold_tile(const FoldArgs<typename CFG::R> &a, int tile, long long boff,
                                           unsigned char *smem_raw)
 {
     using R = typename CFG::R;
@@ -333,6 +377,9 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
 #pragma unroll
         for (int i = 0; i < CFG::EPT; ++i) v[i] = make_cx<R>(v[i].x * f, v[i].y * f);
     }
+    [[maybe_unused]] bool again = false;
+    if constexpr (CFG::CARRIES && !AGAIN) again = may_overflow<CFG::EPT>(v, CFG::LGA + CFG::LGB);
+    if constexpr (AGAIN) __syncthreads();          // the exchange has been read
     if constexpr (TW == 2) {
         if constexpr (CFG::EPT != 32) load_twiddles();
 #pragma unroll
@@ -367,13 +414,15 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
                 for (int r = 1; r < A; ++r) v[u * A + r] = cmul(v[u * A + r], f1(r));
                 plain_dft<A>(v + u * A);
             } else {
-                fold_dft<false, R, A>(v + u * A, f1);
+                fold_dft<AGAIN ? SAFE : CFG::BFLY1, R, A>(v + u * A, f1);
             }
         }
 #pragma unroll
         for (int k = 0; k < A; ++k) ex[FIRST ? k : k * CFG::SK] = v[u * A + k];
     }
-    __syncthreads();
+    // (the answer is asked for after F2, whose table reads would else wait for it)
+    if constexpr (CFG::CARRIES && !AGAIN) again = __syncthreads_or(again);
+    else __syncthreads();
     // ---- F2
 #pragma unroll
     for (int u = 0; u < U2; ++u) {
@@ -391,7 +440,7 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             const V *t2 = reinterpret_cast<const V *>(a.tau);
             if constexpr (TW == 1) t2 += c0 + col + ((unsigned)(CFG::NA + klo) << a.lg_k);
             else t2 += klo;
-            fold_dft<CFG::DIRECT, R, B>(v + u * B, [&](int q) {
+            fold_dft<AGAIN ? SAFE : CFG::BFLY2, R, B>(v + u * B, [&](int q) {
                 const V t = __ldg(t2 + (TW == 1 ? (unsigned)(q * A) << a.lg_k : (unsigned)(q * A)));
                 const C w = make_cx<R>(t.x, t.y);
                 if constexpr (TW != 2) return w;
@@ -400,6 +449,8 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
                 return cmul(w, tabB[lg * W + col]);
             });
         }
+        if constexpr (CFG::CARRIES && !AGAIN)
+            if (u == 0 && again) return true;
         V *q;
         if constexpr (FIRST) {
             const unsigned c = c0 + col;
@@ -428,17 +479,49 @@ __device__ __forceinline__ void fold_tile(const FoldArgs<typename CFG::R> &a, in
             else __stcs(q + a.rowK[k], o);
         }
     }
+    return false;
+}
+
+// The transform's tile and offset of a CTA.  Every second pass takes the tiles
+// from the end: what the pass before it wrote last is still in L2.
+template <typename R>
+__device__ __forceinline__ void fold_cta(const FoldArgs<R> &a, int *tile, long long *boff)
+{
+    const unsigned b = a.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+    *tile = (int)(b & ((1u << a.lg_all) - 1u));
+    *boff = (long long)(b >> a.lg_all) * a.bstride;
+}
+
+// The tile with AGAIN, out of line.
+template <class CFG>
+__device__ __noinline__ void fold_again(const FoldArgs<typename CFG::R> &a, unsigned char *smem_raw)
+{
+    int tile;
+    long long boff;
+    fold_cta(a, &tile, &boff);
+    fold_tile<CFG, false, true>(a, tile, boff, smem_raw);
 }
 
 template <class CFG>
 __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __grid_constant__ FoldArgs<typename CFG::R> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // every second pass takes the tiles from the end: what the pass before it
-    // wrote last is still in L2
     grid_launch_dependents();
-    const unsigned b = a.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
-    fold_tile<CFG, true>(a, (int)(b & ((1u << a.lg_all) - 1u)), (long long)(b >> a.lg_all) * a.bstride, smem_raw);
+    int tile;
+    long long boff;
+    fold_cta(a, &tile, &boff);
+    if (fold_tile<CFG, true>(a, tile, boff, smem_raw)) {
+        if constexpr (CFG::CARRIES) {
+            // (inline where it costs the common path nothing: 8 x 2^24 1010 us for
+            // 1030, but 20 x 2^14, passes of 128 points, 10.2 for 8.2)
+            if constexpr (CFG::LGB < 4) {
+                fold_again<CFG>(a, smem_raw);
+            } else {
+                fold_cta(a, &tile, &boff);
+                fold_tile<CFG, false, true>(a, tile, boff, smem_raw);
+            }
+        }
+    }
 }
 
 // What the host needs to launch one of the kernels above.

@@ -43,27 +43,33 @@ struct WholeSteps {
     }
 };
 
-template <int LG, int EPT, int NT>
+template <int LG_, int EPT, int NT>
 struct WholeCfg {
-    using S = WholeSteps<LG>;
-    static constexpr int N = 1 << LG, TE = EPT * NT, G = TE / N;
+    using S = WholeSteps<LG_>;
+    static constexpr int LG = LG_, N = 1 << LG, TE = EPT * NT, G = TE / N;
     static constexpr int EX0 = G * S::gs(0), EX1 = S::r(2) ? G * S::gs(1) : 0;
     static constexpr int SMEM = (EX0 > EX1 ? EX0 : EX1) * 8;
     static_assert(G >= 1 && S::r(0) <= EPT, "tile");
 };
 
 // Step I of the tile's transforms.  off(g): element offset of transform g, or
-// negative where the tile has none; f multiplies the input.
-template <class CFG, int EPT, int NT, int I, class Off>
-__device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
+// negative where the tile has none; f multiplies the input.  True: nothing was
+// stored, the tile is to be done with AGAIN (may_overflow).
+template <class CFG, int EPT, int NT, int I, bool AGAIN = false, class Off>
+__device__ __forceinline__ bool whole_step(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
                                            const Off &off, cx<float> *sm)
 {
     using S = typename CFG::S;
     using C = cx<float>;
     constexpr int R = S::r(I), K = S::k(I), N = CFG::N, SQ = N / R, U = EPT / R, J = SQ / K;
     constexpr bool LAST = S::r(I + 1) == 0;
+    // Up to 2^7 points the copy rate leaves room for the closer form; above, the
+    // question (may_overflow) costs less: 3001 x 2^12 34.6 -> 35.0 us (DIRECT 35.4),
+    // 200 x 2^13 7.8 -> 8.1 (8.4).
+    constexpr int KIND = AGAIN ? SAFE : N <= 128 ? DIRECT : CARRY;
     const int tid = threadIdx.x;
     C v[EPT];
+    [[maybe_unused]] bool big = false;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const int s = tid + NT * u, g = s / SQ, idx = s % SQ;
@@ -95,10 +101,10 @@ __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool c
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u * R + r] = make_cx<float>(v[u * R + r].x * f, v[u * R + r].y * f);
             }
+            if constexpr (KIND == CARRY) big |= may_overflow<R>(v + u * R, CFG::LG);
             plain_dft<R>(v + u * R);
         } else {
-            // (up to 2^7 points the copy rate leaves room for the closer form)
-            fold_dft<(N <= 128), float, R>(v + u * R, [&](int q) {
+            fold_dft<KIND, float, R>(v + u * R, [&](int q) {
                 const float2 t = __ldg(tau + S::tau(I) + q * K + kap);
                 return make_cx<float>(t.x, t.y);
             });
@@ -122,8 +128,31 @@ __device__ __forceinline__ void whole_step(const float2 *in, float2 *out, bool c
         }
     }
     if constexpr (!LAST) {
-        __syncthreads();
-        whole_step<CFG, EPT, NT, I + 1>(in, out, conj, f, tau, off, sm);
+        if constexpr (I == 0 && KIND == CARRY) {
+            if (__syncthreads_or(big)) return true;
+        } else {
+            __syncthreads();
+        }
+        whole_step<CFG, EPT, NT, I + 1, AGAIN>(in, out, conj, f, tau, off, sm);
+    }
+    return false;
+}
+
+// The tile with AGAIN, out of line: it takes no register of the common path.
+template <class CFG, int EPT, int NT, class Off>
+__device__ __noinline__ void whole_again(const float2 *in, float2 *out, bool conj, float f, const float2 *tau, Off off,
+                                         cx<float> *sm)
+{
+    whole_step<CFG, EPT, NT, 0, true>(in, out, conj, f, tau, off, sm);
+}
+
+// The tile's transforms, again where they may overflow.
+template <class CFG, int EPT, int NT, class Off>
+__device__ __forceinline__ void whole_tile(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
+                                           const Off &off, cx<float> *sm)
+{
+    if (whole_step<CFG, EPT, NT, 0>(in, out, conj, f, tau, off, sm)) {
+        if constexpr (CFG::N > 128) whole_again<CFG, EPT, NT>(in, out, conj, f, tau, off, sm);
     }
 }
 
@@ -144,7 +173,7 @@ __global__ void __launch_bounds__(NT, (EPT == 16 ? 1024 : 512) / NT) paco_whole_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const long long t0 = (long long)blockIdx.x * CFG::G;
     const float f = a.scale ? a.mult * (float)__ldg(a.scale) : a.mult;
-    whole_step<CFG, EPT, NT, 0>(
+    whole_tile<CFG, EPT, NT>(
         a.in, a.out, a.conj != 0, f, a.tau, [&](int g) { return t0 + g < a.batch ? (t0 + g) << LG : -1ll; },
         reinterpret_cast<cx<float> *>(smem_raw));
 }
