@@ -512,9 +512,9 @@ __global__ void __launch_bounds__(CFG::NT, CFG::MINB) paco_fold_kernel(const __g
     fold_cta(a, &tile, &boff);
     if (fold_tile<CFG, true>(a, tile, boff, smem_raw)) {
         if constexpr (CFG::CARRIES) {
-            // (inline where it costs the common path nothing: 8 x 2^24 1010 us for
-            // 1030, but 20 x 2^14, passes of 128 points, 10.2 for 8.2)
-            if constexpr (CFG::LGB < 4) {
+            // (in line for 256 and 512 points, 16 x 2^24 2013 us for 2057; the others
+            // spill for it, one 2^20 10.30 us for 10.01)
+            if constexpr (CFG::LGB != 4) {
                 fold_again<CFG>(a, smem_raw);
             } else {
                 fold_cta(a, &tile, &boff);
