@@ -226,7 +226,9 @@ __host__ __device__ constexpr bool fold_plain(bool fp64, int lgB) { return fp64 
 // EPT_: points a thread holds (0: 16, or 32 where a factor needs them).
 // SCALED_: FIRST with FoldArgs::mult and scale (a kernel of its own: with a branch in
 // the one kernel 23 x 1024^2 went from 145 to 147 us).
-template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0, bool SCALED_ = false>
+// CLOSER_: F2 in the DIRECT form (FP64 routes of three passes and more).
+template <typename R_, int LGA_, int LGB_, int LGW_, bool FIRST_, int TW_, int EPT_ = 0, bool SCALED_ = false,
+          bool CLOSER_ = false>
 struct FoldCfg {
     using R = R_;
     static constexpr int LGA = LGA_, LGB = LGB_, LGW = LGW_;
@@ -256,7 +258,11 @@ struct FoldCfg {
     // 337.9; but 2^28 (512 points, TW 2) 2283, 2385, 2345, and the 2-D form's 1024 points
     // (23 x 1024^2) 144.8, 150.8, 146.4.
     static constexpr int BFLY1 = TW == 2 && EPT == 32 ? DIRECT : CARRY;
-    static constexpr int BFLY2 = TW != 1 && !FP64 ? DIRECT : CARRY;
+    // In FP64 the error decides (relative L2 against a long-double FFT; stage kernels,
+    // CARRY, DIRECT): 2^18 2.90e-16, 2.82, -; but 2^20 3.05e-16, 3.08, 2.97, 2^22 3.18,
+    // 3.22, 3.12, 2^24 3.32, 3.42, 3.29.  From three passes on (TW 2 among them) F2 is
+    // DIRECT: 2^27 21.1 -> 22.5 ms.
+    static constexpr int BFLY2 = CLOSER_ || TW == 2 || (TW == 0 && !FP64) ? DIRECT : CARRY;
     static constexpr bool CARRIES = (TW && !ROWS && BFLY1 == CARRY) || (!PLAIN2 && BFLY2 == CARRY);
     static constexpr int NA = ROWS ? A : A / 2;                   // factors of F1, a column
     static constexpr int NTW = TW == 2 ? (NA + LGB) * W : 0;
@@ -557,6 +563,7 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
 // (the row stride); fn == nullptr where none is built.  scaled: the first pass of a
 // scaled input.
 FoldKernel fold_kernel_f32(bool first, int tw, int lgL, int lgC, bool narrow, bool scaled = false);
-FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC);
+// closer: a later pass of three or more.
+FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC, bool closer);
 
 } // namespace paco

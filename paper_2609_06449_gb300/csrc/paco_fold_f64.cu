@@ -3,10 +3,10 @@
 
 namespace paco {
 
-template <bool FIRST, int TW>
+template <bool FIRST, int TW, bool CLOSER = false>
 static FoldKernel pick(int lgL, int lgC)
 {
-#define PACO_FOLD(LGA, LGB, LGW) (lgC >= LGW ? fold_kernel_of<FoldCfg<double, LGA, LGB, LGW, FIRST, TW>>() : FoldKernel())
+#define PACO_FOLD(LGA, LGB, LGW) (lgC >= LGW ? fold_kernel_of<FoldCfg<double, LGA, LGB, LGW, FIRST, TW, 0, false, CLOSER>>() : FoldKernel())
     switch (lgL) {
     case 5: return PACO_FOLD(4, 1, 5);
     case 6: return PACO_FOLD(3, 3, 4);
@@ -17,10 +17,12 @@ static FoldKernel pick(int lgL, int lgC)
     }
 }
 
-FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC)
+FoldKernel fold_kernel_f64(bool first, int tw, int lgL, int lgC, bool closer)
 {
     if (first) return pick<true, 0>(lgL, lgC);
-    return tw == 0 ? pick<false, 0>(lgL, lgC) : tw == 1 ? pick<false, 1>(lgL, lgC) : pick<false, 2>(lgL, lgC);
+    if (tw == 0) return pick<false, 0>(lgL, lgC);
+    if (tw == 2) return pick<false, 2>(lgL, lgC);
+    return closer ? pick<false, 1, true>(lgL, lgC) : pick<false, 1>(lgL, lgC);
 }
 
 } // namespace paco

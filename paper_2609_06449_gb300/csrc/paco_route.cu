@@ -311,7 +311,7 @@ paco_status_t route_setup(paco_plan *pl)
         const int lgC = i == 0 ? lgN - f[0] : lgK;
         r->twmode[i] = i == 0 || pl->dims >= 2 ? 0 : lgK + f[i] <= DIRECT_LG ? 1 : 2;
         r->k[i] = pl->esize == 8 ? fold_kernel_f32(i == 0, r->twmode[i], f[i], lgC, pl->N * pl->batch <= (int64_t)1 << 24)
-                                 : fold_kernel_f64(i == 0, r->twmode[i], f[i], lgC);
+                                 : fold_kernel_f64(i == 0, r->twmode[i], f[i], lgC, n > 2);
         if (!r->k[i].fn) n = 0;
         if (i == 0 && pl->esize == 8)
             r->scaled = fold_kernel_f32(true, 0, f[i], lgC, pl->N * pl->batch <= (int64_t)1 << 24, true);
