@@ -28,11 +28,20 @@
  *     the forward transform; +1 is this library's reading (the adjoint).
  *
  * Ownership: the caller owns every buffer passed in.  A plan owns its
- * twiddle tables and a device status word; it holds no N-sized scratch (a
- * plan with a 2^14 complex64 factor also owns a 48 MiB ring of L2-resident
- * panel buffers and its counters).
+ * tables of factors and a device status word, and what its two stages need
+ * beside them: a complex64 stage of 2^14 a 48 MiB ring of L2-resident panel
+ * buffers with its counters, one that runs in two passes (stage_split) N * batch
+ * elements.  Where paco_execute runs as passes (paco_plan_info.passes), which
+ * use neither, the stages' part is allocated by the first paco_execute_stage1
+ * or _stage2 call of the plan (or weighted call that runs a stage);
+ * PACO_ERR_NOMEM then leaves the plan usable.
+ * Tables of factors: about K L / 2 entries of the dtype for a pass of L points
+ * after K frequencies up to K L = 2^20, above that 12 to 36 K -- for one plan of
+ * 2^20, 2^24, 2^27, 2^28 points 4, 6, 41, 82 MiB (complex64), 10, 21, 146, 613 MiB
+ * (complex128).
  * Execution entry points enqueue work on `stream` and return without
- * synchronising; they allocate nothing.
+ * synchronising; they allocate nothing but the stages' part above (which a
+ * call recorded by a stream capture may do as well).
  *
  * Errors: every entry point returns a paco_status_t (plan constructors that
  * return a pointer return NULL instead).  On failure a message for the

@@ -283,6 +283,44 @@ static paco_status_t setup_stage(paco_plan *pl, StageCfg *sc, int lgL, int64_t C
     return PACO_OK;
 }
 
+// The scratch of the panel and split stages, once.  paco_execute of a plan with
+// passes touches none of it (16 x 2^24: 2 GiB, 2^14 x 2^14: 48 MiB), so such a plan
+// takes it in its first stage call, which may be one that a graph records: nothing
+// here is enqueued, and the thread's capture mode lets the allocation through.
+static paco_status_t stage_scratch(paco_plan *pl)
+{
+    if (pl->stage_ready.load(std::memory_order_acquire)) return PACO_OK;
+    std::lock_guard<std::mutex> lock(pl->stage_mutex);
+    if (pl->stage_ready.load(std::memory_order_relaxed)) return PACO_OK;
+    size_t scratch_elems = 0, words = 0;
+    for (int k = 0; k < 2; ++k) {
+        const StageCfg &sc = pl->st[k];
+        if (!sc.panel) continue;
+        const int64_t C = (k == 0) ? pl->N2 : pl->N1;
+        scratch_elems = std::max(scratch_elems, (size_t)panel::NBUF * ((size_t)1 << sc.lgL) * sc.P);
+        words = std::max(words, (size_t)(2 * pl->batch * (C / sc.P) + 1));
+    }
+    const bool split = (pl->st[0].split || pl->st[1].split) && pl->batch > 0;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaError_t e = cudaSuccess;
+    const char *what = "panel scratch";
+    if (scratch_elems && !pl->scratch) e = cudaMalloc(&pl->scratch, scratch_elems * pl->esize);
+    if (e == cudaSuccess && scratch_elems && !pl->ctr) e = cudaMalloc((void **)&pl->ctr, words * sizeof(unsigned));
+    if (e == cudaSuccess && split && !pl->split_scratch) {
+        what = "split-stage scratch";
+        e = cudaMalloc(&pl->split_scratch, (size_t)(pl->N * pl->batch) * pl->esize);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();                            // (a later call may find the memory)
+        return fail(PACO_ERR_NOMEM, "%s: %s", what, cudaGetErrorString(e));
+    }
+    pl->ctr_words = words;
+    pl->stage_ready.store(true, std::memory_order_release);
+    return PACO_OK;
+}
+
 static paco_status_t plan_build(paco_plan **out, const paco_plan_opts_t *o, int shard_G = 0, int shard_rank = 0)
 {
     *out = nullptr;
@@ -400,29 +438,9 @@ static paco_status_t plan_build(paco_plan **out, const paco_plan_opts_t *o, int 
         paco_plan_destroy(pl);
         return st;
     }
-    size_t scratch_elems = 0, words = 0;
-    for (int k = 0; k < 2; ++k) {
-        const StageCfg &sc = pl->st[k];
-        if (!sc.panel) continue;
-        const int64_t C = (k == 0) ? pl->N2 : pl->N1;
-        scratch_elems = std::max(scratch_elems, (size_t)panel::NBUF * ((size_t)1 << sc.lgL) * sc.P);
-        words = std::max(words, (size_t)(2 * pl->batch * (C / sc.P) + 1));
-    }
-    if (scratch_elems) {
-        cudaError_t ea = cudaMalloc(&pl->scratch, scratch_elems * pl->esize);
-        if (ea == cudaSuccess) ea = cudaMalloc((void **)&pl->ctr, words * sizeof(unsigned));
-        if (ea != cudaSuccess) {
-            paco_plan_destroy(pl);
-            return fail(PACO_ERR_NOMEM, "panel scratch: %s", cudaGetErrorString(ea));
-        }
-        pl->ctr_words = words;
-    }
-    if ((pl->st[0].split || pl->st[1].split) && pl->batch > 0) {
-        cudaError_t ea = cudaMalloc(&pl->split_scratch, (size_t)(pl->N * pl->batch) * pl->esize);
-        if (ea != cudaSuccess) {
-            paco_plan_destroy(pl);
-            return fail(PACO_ERR_NOMEM, "split-stage scratch: %s", cudaGetErrorString(ea));
-        }
+    if (!route_passes(pl) && (st = stage_scratch(pl)) != PACO_OK) {
+        paco_plan_destroy(pl);
+        return st;
     }
     cudaError_t e = cudaMalloc(&pl->d_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(pl->d_status, 0, sizeof(int));
@@ -714,6 +732,7 @@ extern "C" paco_status_t paco_execute(paco_plan_t *pl, const void *in, void *out
     if (pl->bs) return batched_execute(pl, in, out, dir, s);
     if (pl->fused) return launch_cluster(pl, in, out, dir, nullptr, s);
     if (use_route(pl)) return route_run(pl, in, out, dir, nullptr, s);
+    if ((st = stage_scratch(pl)) != PACO_OK) return st;
     if ((st = launch_stage(pl, pl->st[0], 1, in, out, dir, s)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[1], 2, out, out, dir, s);
 }
@@ -863,6 +882,7 @@ extern "C" paco_status_t paco_execute_weighted_power(paco_plan_t *pl, const void
     t.st_w = w;
     t.st_loss = loss;
     t.st_weighted = out_weighted ? 1 : 0;
+    if (!route_has_power(pl, 0) && (st = stage_scratch(pl)) != PACO_OK) return st;
     st = route_has_power(pl, 0) ? route_power(pl, 0, in, out, dir, t, s)
                                 : launch_stage(pl, pl->st[0], 1, in, out, dir, s);
     if (st != PACO_OK) return st;
@@ -889,6 +909,7 @@ extern "C" paco_status_t paco_execute_weighted_input(paco_plan_t *pl, const void
     t.ld_mult = mult;
     t.ld_on = 1;
     if (use_route(pl) && !w) return route_run(pl, in, out, dir, &t, s);
+    if ((st = stage_scratch(pl)) != PACO_OK) return st;
     if ((st = launch_stage(pl, pl->st[0], 1, in, out, dir, s, &t)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[1], 2, out, out, dir, s);
 }
@@ -900,6 +921,7 @@ extern "C" paco_status_t paco_execute_stage1(paco_plan_t *pl, const void *in, vo
     if (st != PACO_OK || pl->batch == 0) return st;
     if (pl->bs) return fail(PACO_ERR_UNSUPPORTED, "%s takes a single-length plan", "paco_execute_stage1");
     set_device(pl);
+    if ((st = stage_scratch(pl)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[0], 1, in, W, dir, (cudaStream_t)stream);
 }
 
@@ -910,6 +932,7 @@ extern "C" paco_status_t paco_execute_stage2(paco_plan_t *pl, const void *W, voi
     if (st != PACO_OK || pl->batch == 0) return st;
     if (pl->bs) return fail(PACO_ERR_UNSUPPORTED, "%s takes a single-length plan", "paco_execute_stage2");
     set_device(pl);
+    if ((st = stage_scratch(pl)) != PACO_OK) return st;
     return launch_stage(pl, pl->st[1], 2, W, out, dir, (cudaStream_t)stream);
 }
 

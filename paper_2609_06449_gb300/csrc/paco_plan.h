@@ -4,7 +4,9 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
+#include <mutex>
 
 #include "../../include/paco.h"
 
@@ -54,6 +56,10 @@ struct paco_plan {
     int num_sms = 0;
     int form = 0;                  // tensor-core precision form (paco_tc.cuh), 0 = plain
     int req_ctas = 0;              // requested CTAs per SM of the stage kernels (0 = default)
+    // what only the stage pipeline needs (scratch, ctr, split_scratch): with the plan
+    // where paco_execute runs the stages, else from the first stage call on
+    std::atomic<bool> stage_ready{false};
+    std::mutex stage_mutex;
     int req_split = 0;             // paco_plan_opts_t.split
     int req_tile = 0;              // 1: a tile width or cluster size was asked for
     paco::Route *route = nullptr;  // the passes of paco_execute (paco_route.cu), or nullptr: the stage kernels
