@@ -411,18 +411,8 @@ static paco_status_t plan_build(paco_plan **out, const paco_plan_opts_t *o, int 
         paco_plan_destroy(pl);
         return st;
     }
-    // FP64-generated twiddle tables: w_N1^{-r}, w_N2^{-r}, and w_N^{-r} in
-    // two levels (r = hi * 2^h + lo).  The 2-D DFT has no top-level twiddle:
-    // its w_N tables are w_1 = 1 (every kernel then multiplies by one).
-    const int lgN = l1 + l2;
-    pl->twN_lo_bits = (lgN + 1) / 2;
-    const long long nlo = 1LL << pl->twN_lo_bits, nhi = (1LL << lgN) / nlo;
-    const long long Mtw = (pl->dims >= 2) ? 1 : pl->N;
-    if ((st = gen_table(pl->esize, &pl->twL1, pl->N1, pl->N1, 1, 0)) != PACO_OK ||
-        (st = gen_table(pl->esize, &pl->twL2, pl->N2, pl->N2, 1, 0)) != PACO_OK ||
-        (st = gen_table(pl->esize, &pl->twN_lo, Mtw, nlo, 1, 0)) != PACO_OK ||
-        (st = gen_table(pl->esize, &pl->twN_hi, Mtw, nhi, nlo, 0)) != PACO_OK ||
-        (pl->dims == 3 && (st = gen_table(pl->esize, &pl->tw_ones, 1, pl->N2, 1, 0)) != PACO_OK)) {
+    // (generated in FP64; the weighted power is complex64's, in one and two dimensions)
+    if ((st = plan_tables(pl, pl->dtype == PACO_C64 && pl->dims != 3)) != PACO_OK) {
         paco_plan_destroy(pl);
         return st;
     }
@@ -477,12 +467,8 @@ extern "C" void paco_plan_destroy(paco_plan_t *pl)
     route_destroy(pl->route);
     restore_destroy(pl);
     cudaFree(pl->tc);
-    cudaFree(pl->twL1);
-    cudaFree(pl->twL2);
-    cudaFree(pl->twN_lo);
-    cudaFree(pl->twN_hi);
+    cudaFree(pl->tables);
     cudaFree(pl->cluster_tau);
-    cudaFree(pl->tw_ones);
     cudaFree(pl->split_scratch);
     for (int k = 0; k < 2; ++k)
         for (int p = 0; p < 2; ++p) cudaFree(pl->st[k].sp_tw[p]);

@@ -340,17 +340,12 @@ paco_status_t cluster_setup(paco_plan *pl)
     // the factors of two passes of 16 x 16 points, in one table
     FoldKernel k;
     k.lgA = k.lgB = 4;
-    void *t1 = nullptr, *t2 = nullptr;
-    paco_status_t st = fold_table<float>(&t1, k, 0, 0);
-    if (st == PACO_OK) st = fold_table<float>(&t2, k, 1, 8, pl->dims >= 2);   // (the 2-D DFT has no top-level twiddle)
-    cudaError_t e = cudaSuccess;
-    if (st == PACO_OK && (e = cudaMalloc(&pl->cluster_tau, (128 + 136 * 256) * sizeof(float2))) == cudaSuccess &&
-        (e = cudaMemcpy(pl->cluster_tau, t1, 128 * sizeof(float2), cudaMemcpyDeviceToDevice)) == cudaSuccess)
-        e = cudaMemcpy(static_cast<float2 *>(pl->cluster_tau) + 128, t2, 136 * 256 * sizeof(float2), cudaMemcpyDeviceToDevice);
-    cudaFree(t1);
-    cudaFree(t2);
-    if (st == PACO_OK && e != cudaSuccess) st = fail(PACO_ERR_CUDA, "one-launch form: %s", cudaGetErrorString(e));
-    return st;
+    const paco_status_t st = fold_table<float>(&pl->cluster_tau, k, 1, 8, pl->dims >= 2,    // (the 2-D DFT has no top-level twiddle)
+                                               128 * sizeof(float2));
+    if (st != PACO_OK) return st;
+    fold_levels(pl->cluster_tau, k);
+    PACO_CUDA_TRY(cudaGetLastError());
+    return PACO_OK;
 }
 
 } // namespace paco

@@ -555,9 +555,12 @@ template <typename R>
 void fold_pass_args(FoldArgs<R> *a, const FoldKernel &k, const int *f, int n, int i, int t);
 
 // A device table for FoldArgs::tau in mode FoldCfg::TW, 2^lgK columns.
-// kappa = 0 for every column where no_kappa is set.
+// kappa = 0 for every column where no_kappa is set.  The first `skip` bytes of
+// *dst (a multiple of 16) are left to the caller.
 template <typename R>
-paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa = false);
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa = false, size_t skip = 0);
+// The complex64 table of mode 0 (2^(lgL - 1) factors of F2) at dst.
+void fold_levels(void *dst, const FoldKernel &k);
 
 // The kernel for a pass of length 2^lgL whose row blocks have 2^lgC columns
 // (the row stride); fn == nullptr where none is built.  scaled: the first pass of a

@@ -47,7 +47,9 @@ struct paco_plan {
     int device = 0;
     paco::StageCfg st[2];          // stage 1 (L = N1, C = N2), stage 2 (L = N2, C = N1)
     paco::StageCfg ph1;            // Phase I alone (mode 3), same geometry as st[0]
+    void *tables = nullptr;        // one allocation (plan_tables), which holds
     void *twL1 = nullptr, *twL2 = nullptr, *twN_lo = nullptr, *twN_hi = nullptr;
+    void *twP[2] = {nullptr, nullptr};     // the weighted power's w_L1^{-r}, w_L2^{-r}
     int twN_lo_bits = 0;
     int *d_status = nullptr;
     void *scratch = nullptr;       // panel ring buffers (L2-sized, not N-sized)
@@ -90,6 +92,11 @@ int ilog2_exact(int64_t v);
 // FP64-generated table of w_M^{-(r*mult)}, r in [count], complex of `esize` bytes
 paco_status_t gen_table(int esize, void **dst, long long M, long long count, long long mult,
                         cudaStream_t stream);
+
+// paco_power.cu: the plan's tables of roots of N1, N2 and N (the 2-D and 3-D DFT
+// have no top-level twiddle: ones), in one allocation and one launch (four of each
+// took 30 us more); power: those of the weighted power too.
+paco_status_t plan_tables(paco_plan *pl, bool power);
 
 // paco_stage_tc.cu
 const void *stage_kernel_fn_tc(int lgL, int form);

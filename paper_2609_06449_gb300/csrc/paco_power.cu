@@ -34,18 +34,64 @@ static PowerKernel pick(int lgL, int lgC)
     }
 }
 
-__global__ void power_table_kernel(const cx<float> *w, cx<float> *out, int lgL)
+// Entry r < count: w_M^{-r mult}, or (split) the product of entries r mod split and
+// the rest of r, as the weighted power's stages take it.
+struct TableSpec {
+    void *out;
+    long long M, mult;
+    int count, split;
+};
+struct TableSpecs {
+    TableSpec t[7];
+};
+template <typename R>
+__global__ void plan_tables_kernel(const __grid_constant__ TableSpecs specs)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x, s = 1 << ((lgL + 1) / 2);
-    if (r >= 1 << lgL) return;
-    const cx<float> lo = w[r & (s - 1)], hi = w[r & ~(s - 1)];
-    out[r] = lgL > 6 ? st::mul<1>(lo, hi) : st::mul<0>(lo, hi);
+    const TableSpec &t = specs.t[blockIdx.y];
+    auto root = [&](long long r) {
+        double sn, cs;
+        sincospi(2.0 * (double)((r * t.mult) % t.M) / (double)t.M, &sn, &cs);
+        return make_cx<R>((R)cs, (R)(-sn));
+    };
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < t.count; r += gridDim.x * blockDim.x) {
+        cx<R> w = root(t.split ? r & (t.split - 1) : r);
+        if constexpr (sizeof(R) == 4)
+            if (t.split) {
+                const cx<R> hi = root(r & ~(t.split - 1));
+                w = t.count > 64 ? st::mul<1>(w, hi) : st::mul<0>(w, hi);
+            }
+        static_cast<cx<R> *>(t.out)[r] = w;
+    }
 }
 
-paco_status_t power_table(const cx<float> *w, int lgL, void **dst)
+paco_status_t plan_tables(paco_plan *pl, bool power)
 {
-    PACO_CUDA_TRY(cudaMalloc(dst, (size_t)8 << lgL));
-    power_table_kernel<<<((1 << lgL) + 255) / 256, 256>>>(w, static_cast<cx<float> *>(*dst), lgL);
+    const int lgN = ilog2_exact(pl->N);
+    pl->twN_lo_bits = (lgN + 1) / 2;
+    const long long nlo = 1LL << pl->twN_lo_bits, nhi = pl->N / nlo, Mtw = pl->dims >= 2 ? 1 : pl->N;
+    auto split = [](int64_t L) { return 1 << ((ilog2_exact(L) + 1) / 2); };
+    struct { void **dst; TableSpec t; } want[7] = {
+        {&pl->twL1, {nullptr, pl->N1, 1, (int)pl->N1, 0}},
+        {&pl->twL2, {nullptr, pl->N2, 1, (int)pl->N2, 0}},
+        {&pl->twN_lo, {nullptr, Mtw, 1, (int)nlo, 0}},
+        {&pl->twN_hi, {nullptr, Mtw, nlo, (int)nhi, 0}},
+        {&pl->tw_ones, {nullptr, 1, 1, pl->dims == 3 ? (int)pl->N2 : 0, 0}},
+        {&pl->twP[0], {nullptr, pl->N1, 1, power ? (int)pl->N1 : 0, split(pl->N1)}},
+        {&pl->twP[1], {nullptr, pl->N2, 1, power ? (int)pl->N2 : 0, split(pl->N2)}}};
+    size_t bytes = 0;
+    TableSpecs specs;
+    int n = 0;
+    for (auto &w : want) bytes += ((size_t)w.t.count * pl->esize + 255) & ~(size_t)255;
+    PACO_CUDA_TRY(cudaMalloc(&pl->tables, bytes));
+    bytes = 0;
+    for (auto &w : want) {
+        if (!w.t.count) continue;
+        w.t.out = *w.dst = static_cast<char *>(pl->tables) + bytes;
+        specs.t[n++] = w.t;
+        bytes += ((size_t)w.t.count * pl->esize + 255) & ~(size_t)255;
+    }
+    if (pl->esize == 8) plan_tables_kernel<float><<<dim3(64, n), 256>>>(specs);
+    else plan_tables_kernel<double><<<dim3(64, n), 256>>>(specs);
     PACO_CUDA_TRY(cudaGetLastError());
     return PACO_OK;
 }

@@ -29,7 +29,7 @@ struct PowerArgs {
     int rev_bits, rev_t;    // row map of j_lo: pi over rev_bits bits (0: natural rows)
     int crev_bits, crev_t;  // Phase I: row pi(c) of column c
     int lg_all;             // log2 of the tiles of one transform (blockIdx.x = transform, tile)
-    const cx<float> *twL;   // w_L^{-r}, r < L, as the stage kernels' product of two factors (power_table)
+    const cx<float> *twL;   // w_L^{-r}, r < L, as the stage kernels' product of two factors (plan_tables)
     const cx<float> *lo;    // w_N^{-r}, r < 2^lo_bits
     const cx<float> *hi;    // w_N^{-(r << lo_bits)}
     int lo_bits;
@@ -307,9 +307,5 @@ struct PowerKernel {
 // The kernel of a stage of length 2^lgL over 2^lgC columns; fn == nullptr
 // where none is built.
 PowerKernel power_kernel(bool first, int lgL, int lgC);
-
-// PowerArgs::twL from w_L^{-r} (r < L = 2^lgL): entry r is the product
-// w[r mod S] w[r / S * S], S = 2^ceil(lgL / 2), that the stage kernels take.
-paco_status_t power_table(const cx<float> *w, int lgL, void **dst);
 
 } // namespace paco

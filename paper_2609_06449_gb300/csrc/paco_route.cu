@@ -38,7 +38,7 @@ struct Route {
     TcPassArgs t[MAX_PASSES];
     PowerKernel pk[2];              // the stages of the weighted power (fn == nullptr: the stage kernels)
     PowerArgs pa[2];
-    void *tw[MAX_PASSES + 2] = {};     // the factors of every pass, w_L^{-r} of the two stages
+    void *tw[MAX_PASSES] = {};         // the factors of every pass
 };
 
 // pi over `bits` bits with digits of t bits (host copy of digit_reverse).
@@ -112,19 +112,25 @@ static cx<R> *tau_gen(cx<R> *t, int entries, int kind, int lgA, int lgK, bool no
     return t + count;
 }
 
-// FoldArgs::tau in mode FoldCfg::TW over 2^lgK columns.
+// Entries of FoldArgs::tau in mode FoldCfg::TW over 2^lgK columns.
+static long long fold_entries(bool fp64, const FoldKernel &k, int mode, int lgK)
+{
+    const int A = 1 << k.lgA, B = 1 << k.lgB, nA = fp64 ? A : A / 2;
+    if (mode == 0 && fold_plain(fp64, k.lgB)) return A * B;
+    return mode == 1 ? (long long)(nA + A * B / 2) << lgK : A * B / 2 + (mode == 2 ? (long long)(nA + k.lgB) << lgK : 0);
+}
+
 template <typename R>
-paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa)
+paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, bool no_kappa, size_t skip)
 {
     const int A = 1 << k.lgA, B = 1 << k.lgB, lgL = k.lgA + k.lgB;
     const bool fp64 = sizeof(R) == 8;
     if (mode == 0 && fold_plain(fp64, k.lgB)) return gen_table((int)sizeof(cx<R>), dst, A * B, A * B, 1, 0);
     const int nA = fp64 ? A : A / 2;
-    const long long cols = 1ll << lgK;
-    const long long count = mode == 1 ? (nA + A * B / 2) * cols : A * B / 2 + (mode == 2 ? (nA + k.lgB) * cols : 0);
+    const long long count = fold_entries(fp64, k, mode, lgK);
     // FP32 tables of many entries: FP64 roots of w_{K L} behind the table
     Roots roots;
-    size_t bytes = ((size_t)count * sizeof(cx<R>) + 15) & ~(size_t)15;
+    size_t bytes = skip + (((size_t)count * sizeof(cx<R>) + 15) & ~(size_t)15);
     const bool by_roots = !fp64 && mode != 0 && !no_kappa;
     if (by_roots) {
         roots.lg = lgK + lgL;
@@ -138,7 +144,7 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
         roots.lo = q;
         roots.hi = q + (1 << roots.lo_bits);
     }
-    cx<R> *t = static_cast<cx<R> *>(*dst);
+    cx<R> *t = reinterpret_cast<cx<R> *>(static_cast<char *>(*dst) + skip);
     if (mode == 1) {
         t = fp64 ? tau_gen(t, A, TAU_ROWS, k.lgA, lgK, no_kappa) : tau_gen(t, nA, TAU_LEVELS, 0, lgK, no_kappa, roots);
         tau_gen(t, A * B / 2, TAU_LEVELS, k.lgA, lgK, no_kappa, roots);
@@ -153,7 +159,9 @@ paco_status_t fold_table(void **dst, const FoldKernel &k, int mode, int lgK, boo
     return PACO_OK;
 }
 
-template paco_status_t fold_table<float>(void **, const FoldKernel &, int, int, bool);
+template paco_status_t fold_table<float>(void **, const FoldKernel &, int, int, bool, size_t);
+
+void fold_levels(void *dst, const FoldKernel &k) { tau_gen(static_cast<cx<float> *>(dst), 1 << (k.lgA + k.lgB - 1), TAU_LEVELS, k.lgA, 0); }
 
 paco_status_t whole_table(int lgN, void **dst)
 {
@@ -211,7 +219,7 @@ static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, c
 }
 
 // Stage i of the weighted power over the plan's factors.
-static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerKernel &k, void **tw, const int *lg, int i)
+static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerKernel &k, const int *lg, int i)
 {
     memset(a, 0, sizeof(*a));
     const int lgL = lg[i], lgC = lg[1 - i];
@@ -229,9 +237,8 @@ static paco_status_t power_setup(const paco_plan *pl, PowerArgs *a, const PowerK
     a->lo_bits = pl->twN_lo_bits;
     a->n_mask = (unsigned)(pl->N - 1);
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    const paco_status_t st = power_table(static_cast<const cx<float> *>(i == 0 ? pl->twL1 : pl->twL2), lgL, tw);
-    a->twL = static_cast<const cx<float> *>(*tw);
-    return st;
+    a->twL = static_cast<const cx<float> *>(pl->twP[i]);
+    return PACO_OK;
 }
 
 // Factors of the route, log2, first pass first; returns their number (0: none).
@@ -329,7 +336,7 @@ paco_status_t route_setup(paco_plan *pl)
     if (pl->dims == 3 || pl->esize != 8) return st;
     for (int i = 0; i < 2 && st == PACO_OK; ++i) {
         r->pk[i] = power_kernel(i == 0, lg[i], lg[1 - i]);
-        if (r->pk[i].fn) st = power_setup(pl, &r->pa[i], r->pk[i], &r->tw[MAX_PASSES + i], lg, i);
+        if (r->pk[i].fn) st = power_setup(pl, &r->pa[i], r->pk[i], lg, i);
     }
     return st;
 }
