@@ -38,7 +38,8 @@
  * Tables of factors: about K L / 2 entries of the dtype for a pass of L points
  * after K frequencies up to K L = 2^20, above that 12 to 36 K -- for one plan of
  * 2^20, 2^24, 2^27, 2^28 points 4, 6, 41, 82 MiB (complex64), 10, 21, 146, 613 MiB
- * (complex128).
+ * (complex128).  The plans of a process that need the same table on a device hold
+ * it together; it is freed with the last of them.
  * Execution entry points enqueue work on `stream` and return without
  * synchronising; they allocate nothing but the stages' part above (which a
  * call recorded by a stream capture may do as well).

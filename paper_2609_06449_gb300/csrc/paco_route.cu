@@ -11,7 +11,11 @@
 // plan's own two stages (paco_power.cuh).
 #include <cuda_runtime.h>
 
+#include <array>
 #include <cstring>
+#include <map>
+#include <memory>
+#include <mutex>
 #include <new>
 
 #include "paco_common.cuh"
@@ -38,7 +42,7 @@ struct Route {
     TcPassArgs t[MAX_PASSES];
     PowerKernel pk[2];              // the stages of the weighted power (fn == nullptr: the stage kernels)
     PowerArgs pa[2];
-    void *tw[MAX_PASSES] = {};         // the factors of every pass
+    std::shared_ptr<void> tw[MAX_PASSES];   // the factors of every pass (shared_table)
 };
 
 // pi over `bits` bits with digits of t bits (host copy of digit_reverse).
@@ -49,10 +53,35 @@ static unsigned rev_host(unsigned u, int bits, int t)
 
 void route_destroy(Route *r)
 {
-    if (!r) return;
-    for (void *p : r->tw) cudaFree(p);
     delete r;
 }
+
+// A table of factors, one for all plans that are alive on a device and need the
+// same one: it depends on the lengths alone, and a program keeps a plan for every
+// batch size and stream that it meets.  key: what tells the tables apart (the
+// device and the kind among it).  make(&p) allocates and enqueues; every plan waits
+// for the device before it is handed out, so a table found here is complete by
+// then whichever plan made it.  Freed with the last plan that holds it.
+using TableKey = std::array<int, 7>;
+template <class Make>
+static paco_status_t shared_table(const TableKey &key, std::shared_ptr<void> *out, const Make &make)
+{
+    static std::mutex &mutex = *new std::mutex;        // (not torn down before the last plan)
+    static auto &tables = *new std::map<TableKey, std::weak_ptr<void>>;
+    std::lock_guard<std::mutex> lock(mutex);
+    std::weak_ptr<void> &known = tables[key];
+    if ((*out = known.lock())) return PACO_OK;
+    void *p = nullptr;
+    const paco_status_t st = make(&p);
+    if (st != PACO_OK) {
+        cudaFree(p);
+        return st;
+    }
+    *out = std::shared_ptr<void>(p, [](void *q) { cudaFree(q); });
+    known = *out;
+    return PACO_OK;
+}
+enum { TABLE_FOLD, TABLE_WHOLE, TABLE_ROOTS };
 
 // Tables of a pass's factors, each rounded once, over K = 2^lgK columns (kappa).
 enum TauKind {
@@ -213,8 +242,10 @@ static paco_status_t pass_setup(const paco_plan *pl, Route *r, FoldArgs<R> *a, c
     const FoldKernel &k = r->k[i];
     fold_pass_args(a, k, f, n, i, t);
     PACO_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
-    const paco_status_t st = fold_table<R>(&r->tw[i], k, r->twmode[i], a->lg_k);
-    a->tau = static_cast<const cx<R> *>(r->tw[i]);
+    const int lgK = r->twmode[i] ? a->lg_k : 0;             // (mode 0: one column)
+    const paco_status_t st = shared_table({pl->device, TABLE_FOLD, (int)sizeof(R), k.lgA, k.lgB, r->twmode[i], lgK}, &r->tw[i],
+                                          [&](void **p) { return fold_table<R>(p, k, r->twmode[i], lgK); });
+    a->tau = static_cast<const cx<R> *>(r->tw[i].get());
     return st;
 }
 
@@ -284,9 +315,10 @@ static paco_status_t tc_setup(paco_plan *pl, Route *r, int lgN)
         a.hi = static_cast<const cx<float> *>(pl->twN_hi);
         a.frag = static_cast<const uint4 *>(pl->tc);
         PACO_CUDA_TRY(cudaFuncSetAttribute(r->k[i].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->k[i].smem));
-        const paco_status_t st = gen_table(8, &r->tw[i], 1LL << f[i], 1LL << f[i], 1, 0);
+        const paco_status_t st = shared_table({pl->device, TABLE_ROOTS, 8, f[i], 0, 0, 0}, &r->tw[i],
+                                              [&](void **p) { return gen_table(8, p, 1LL << f[i], 1LL << f[i], 1, 0); });
         if (st != PACO_OK) return st;
-        a.twL = static_cast<const cx<float> *>(r->tw[i]);
+        a.twL = static_cast<const cx<float> *>(r->tw[i].get());
     }
     r->n = n;
     return PACO_OK;
@@ -308,7 +340,8 @@ paco_status_t route_setup(paco_plan *pl)
     // them 8.5 and 8.4, 100 8.6 and 10.9)
     const bool whole = pl->dims == 1 && pl->esize == 8 && (lgN < 13 || pl->batch >= 32);
     if (whole && (r->whole = whole_kernel(lgN)).fn) {
-        const paco_status_t st = whole_table(lgN, &r->tw[0]);
+        const paco_status_t st = shared_table({pl->device, TABLE_WHOLE, 8, lgN, 0, 0, 0}, &r->tw[0],
+                                              [&](void **p) { return whole_table(lgN, p); });
         if (st != PACO_OK) return st;
         PACO_CUDA_TRY(cudaFuncSetAttribute(r->whole.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->whole.smem));
         r->n = 1;
@@ -398,7 +431,7 @@ paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir,
         a.in = static_cast<const float2 *>(in);
         a.out = static_cast<float2 *>(out);
         a.batch = pl->batch;
-        a.tau = static_cast<const float2 *>(r.tw[0]);
+        a.tau = static_cast<const float2 *>(r.tw[0].get());
         a.conj = dir == 1;
         a.mult = terms ? terms->ld_mult : 1.f;
         a.scale = terms ? terms->ld_scale : nullptr;
