@@ -331,8 +331,8 @@ __device__ __forceinline__ bool fold_tile(const FoldArgs<typename CFG::R> &a, in
     const long long base = boff + (long long)blk * (FIRST ? 0u : a.blk_stride) + c0;
 
     // TW 2: the columns' factors.  With 32 points a thread their reads go out
-    // before the tile's (1024 points 0.93 -> 0.87 ms per 2^28, 512: 0.78 -> 0.75);
-    // with 16 they would hold up too many small tiles (256: 0.65, 0.68).
+    // before the tile's (512 points 0.78 -> 0.75 ms per 2^28); with 16 they would hold
+    // up too many small tiles (256: 0.65, 0.68).
     constexpr int NI = (CFG::NTW + NT - 1) / NT;
     [[maybe_unused]] V twl[NI ? NI : 1];
     [[maybe_unused]] auto load_twiddles = [&] {

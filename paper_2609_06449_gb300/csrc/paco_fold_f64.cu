@@ -3,10 +3,20 @@
 
 namespace paco {
 
+// Built: the lengths that a route has in each mode (2^5..2^9; from three passes on
+// 2^6, and 2^7 with TW 2).
+template <bool FIRST, int TW, bool CLOSER, int LGA, int LGB, int LGW>
+static FoldKernel kernel_of(int lgC)
+{
+    if constexpr (LGA + LGB >= (TW == 2 ? 7 : CLOSER ? 6 : 5))
+        if (lgC >= LGW) return fold_kernel_of<FoldCfg<double, LGA, LGB, LGW, FIRST, TW, 0, false, CLOSER>>();
+    return FoldKernel();
+}
+
 template <bool FIRST, int TW, bool CLOSER = false>
 static FoldKernel pick(int lgL, int lgC)
 {
-#define PACO_FOLD(LGA, LGB, LGW) (lgC >= LGW ? fold_kernel_of<FoldCfg<double, LGA, LGB, LGW, FIRST, TW, 0, false, CLOSER>>() : FoldKernel())
+#define PACO_FOLD(LGA, LGB, LGW) kernel_of<FIRST, TW, CLOSER, LGA, LGB, LGW>(lgC)
     switch (lgL) {
     case 5: return PACO_FOLD(4, 1, 5);
     case 6: return PACO_FOLD(3, 3, 4);
