@@ -21,7 +21,7 @@ input as context.
 Other workloads (--workload): A (2^16 as 256 x 256, latency: one cluster
 launch), B128 (complex128 N = 2^27), C (the uneven batch in one persistent
 launch), D (16 x 2^24 per precision form), E (forward + backward of
-256 x 2^20 with the weighted power loss fused into the stage kernels), T
+256 x 2^20 with the weighted power loss fused into its transforms), T
 (the 128-point sub-pass of a 2^14 stage on the tcgen05 tensor cores against
 the plain FP32 kernel), U (the unfused three-pass pipeline Phase I ->
 paco_permute -> Phase III on the headline transform: the ablation of the
@@ -372,7 +372,7 @@ def tc_split(paco, x, y, N1, N2, b, p, K, warmup, stream, flop, world, max_over_
         pl.check()
         ms = max_over_ranks(tot) / KT
         res[name] = {"ms_per_step": ms, "value": flop * world / (ms * 1e-3) / 1e9, "unit": "GFLOP/s",
-                     "steps": KT, "kernel": "paco_stage_kernel, radix-16 passes as mma.sync contractions"}
+                     "steps": KT, "kernel": "paco_tcpass_kernel, radix-16 sub-DFTs as mma.sync contractions"}
         torch_sync()
         outs[name] = y.cpu().numpy()
         pl.close()
@@ -520,7 +520,7 @@ def run_other(args, ranks, local):
                             "input": "Re, Im i.i.d. U[-1,1), seed = rank",
                             "l2": "input fits in L2: latency-bound by design, no flush"},
                     roofline=dict(hbm_roofline("paco_cluster_kernel (one launch, 16-CTA cluster)" if fused
-                                               else "stage kernels (2 launches)",
+                                               else "paco_fold_kernel (2 passes)",
                                                (16.0 if fused else 32.0) * N, statistics.median(per)),
                                   bound="latency"),
                     gflops=5.0 * N * 16 / (us * 1e-6) / 1e9, accuracy=acc,
@@ -858,14 +858,15 @@ def run_other(args, ranks, local):
                     higher_is_better=True, ms_per_step=ms, dtype="f32",
                     config={"workload": "256 x c64 1-D DFT N=2^20 (1024 x 1024, b=4): loss = sum(w |FFT(x)|^2), "
                                         "forward + backward (conjugate transform) through torch.autograd, "
-                                        "the loss and its backward fused into the stage kernels",
+                                        "the loss fused into the forward's stages, its backward into the "
+                                        "passes of the conjugate transform",
                             "input": "x Re, Im i.i.d. N(0,1); w U[0,1)", "l2": "inputs larger than L2"},
                     accuracy=acc,
                     context=dict(cufft_context(x.detach(), N, B, flop / 2),
                                  unfused_ms_per_step=mor(tot_u) / min(K, 20),
                                  unfused="PacoFFT + the loss and its gradient as PyTorch element-wise ops"),
-                    roofline=hbm_roofline("stage kernels (4 launches; w read by the loss epilogue and the "
-                                          "backward's loads)", (4 * 16.0 + 2 * 4.0) * N * B, ms),
+                    roofline=hbm_roofline("paco_power_kernel, paco_fold_kernel (4 launches; w read by the loss "
+                                          "epilogue)", (4 * 16.0 + 4.0) * N * B, ms),
                     e2e=e2e, cpu_baseline=cpu_leg(args, rank, world, lg=20), gpu_launches=4 * K, clocks=clocks)
     if rank == 0:
         emit(line)

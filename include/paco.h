@@ -150,9 +150,10 @@ typedef struct {
                                     pipeline's second factor N2 N3) */
     int64_t N3;                  /* dims = 3: the third axis; 1 otherwise */
     int passes;                  /* launches of paco_execute when it runs as passes over
-                                    factors of N chosen for the machine (plain complex64
-                                    plans with no stage option set); 0: the two stages
-                                    described above */
+                                    factors of N chosen for the machine (plans of every
+                                    dtype with no stage option set, where the kernels are
+                                    built for the lengths); 0: the one-launch form
+                                    (fused_cluster) or the two stages described above */
 } paco_plan_info_t;
 
 /*
@@ -192,10 +193,14 @@ paco_status_t paco_plan_info(const paco_plan_t *plan, paco_plan_info_t *info);
  * to four passes, the first with the redistribution in its stores, the others
  * in place in `out`); the others run the plan's own two stages, W = Z-hat
  * (Eq. (17)) between them.  The launches may be programmatically dependent:
- * they wait for the preceding kernels before they touch `in` or `out`.  in == out, or overlapping buffers, return PACO_ERR_ALIASING.
+ * they wait for the preceding kernels before they touch `in` or `out`.  The
+ * kernels, and with them the last bits of a result, may depend on the batch
+ * (complex64 of 2^13 and 2^14 points: whole transforms from a batch of 32 on).
+ * A sum above the largest number is infinite or NaN in the results it is part of;
+ * results whose own sums stay below are not touched by it.
+ * in == out, or overlapping buffers, return PACO_ERR_ALIASING.
  * batch = 0 is a no-op.  Asynchronous on `stream`.  A complex64 plan with
- * N1 = N2 = 256, p = 4 or 8 and batch <= 16 (where one launch is faster than
- * two) runs as ONE launch (paco_plan_info.fused_cluster): a thread-block
+ * N1 = N2 = 256, p = 4 or 8 and batch <= 16 runs as ONE launch (paco_plan_info.fused_cluster): a thread-block
  * cluster of K = 16 CTAs per transform (8 where the GPU cannot host a
  * 16-CTA cluster), processor q of Sect. 2 being the K/p CTAs that hold its
  * slab -- Phase I on the input columns in shared memory, then PARA-CO-DRP_b

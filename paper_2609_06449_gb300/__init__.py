@@ -233,7 +233,7 @@ def _current_stream(dev: int | None = None) -> int:
     """The raw handle of torch's current stream on ``dev`` (default: the
     current device).  Asked of torch's C layer where it offers that: 0.1 us
     against 2 us for a ``torch.cuda.Stream`` object, of the 7 us that
-    ``Plan.execute`` took on the host (2.7 us now)."""
+    ``Plan.execute`` took on the host (3.5 us now)."""
     import torch
     if dev is None:
         dev = torch.cuda.current_device()
@@ -500,7 +500,7 @@ try:
             return fft(g.contiguous(), N1, N2, b, p, dir=+1), None, None, None, None
     class PacoWeightedPowerLoss(_torch.autograd.Function):
         """loss = sum(w |F x|^2) over the whole batch (float64 scalar), F the
-        paper's forward transform.  Forward: the two stage kernels, the loss
+        paper's forward transform.  Forward: the transform's two stages, the loss
         summed by the Phase III kernel, which stores u = w ⊙ F x (y itself is
         not returned).  Backward: grad_x = F^H (2 g u), the scalar 2 g applied
         as the conjugate transform's Phase I loads its input.  w (float32, the

@@ -1,9 +1,11 @@
 // paco_capi.cu -- host side of the C ABI declared in include/paco.h.
 //
 // Plan construction (legality per Sect. 2, Eq. exact-divisibility; tile and
-// cluster choice; FP64 twiddle tables generated on the device), execution
-// (two stage launches per Theorem 3's composition, Eq. (10)), the unfused
-// three-pass form, the host-buffer form, and error reporting.
+// cluster choice; what the stages need), execution (paco_execute by the passes of
+// paco_route.cu or the one-launch form of paco_cluster.cu, else the two stage
+// launches of Theorem 3's composition, Eq. (10); the stage, weighted and sharded
+// entry points), the unfused three-pass form, the host-buffer form, and error
+// reporting.
 #include <cuda.h>            // CUtensorMap types (no libcuda link: the encoder comes
 #include <cudaTypedefs.h>    // from cudaGetDriverEntryPointByVersion)
 #include <cuda_runtime.h>

@@ -25,7 +25,8 @@
 // The blocks travel as one bulk copy each (2 KiB for K = 16), which counts its
 // bytes on the destination's transaction barrier.  Item by item (st.async of 8
 // bytes) the exchange kept each SM's port busy for 4096 packets a side: the
-// transform took 6.7 us in a replayed graph, and takes 6.05 us so.
+// transform took 6.7 us in a replayed graph, and 6.05 us so (4.3 with the folded
+// butterflies as well).
 // Synchronisation: one split cluster barrier (arrive at entry, wait before the
 // first copy) makes sure every CTA of the cluster runs and has set up its
 // barrier; a CTA starts Phase III as soon as its own N/K items have landed; a
@@ -242,10 +243,11 @@ const void *cluster_kernel_fn(int K)
 }
 
 // The one-launch form applies to complex64 plans with N1 = N2 = 256 and p = 4
-// or 8, up to 16 transforms: it keeps one transform on one cluster of K SMs,
-// which is latency-bound, and from 32 transforms on the two stage launches,
-// which stream the whole batch through all SMs, take less time (measured on
-// GB300: 15.8 vs 16.5 us at 16 transforms, 24.8 vs 21.5 us at 32).
+// or 8, up to 16 transforms.  It keeps one transform on one cluster of K SMs, which
+// is latency-bound; the alternative is two passes over all SMs.  us in a replayed
+// graph, this form and the passes: 1 transform 4.3 and 4.9, 4 4.4 and 5.2, 8 6.8 and
+// 6.4, 12 7.2 and 10.0, 16 9.9 and 10.6.  (The limit of 16 dates from the stage
+// launches before the passes, which were faster at 32.)
 bool cluster_eligible(const paco_plan *pl)
 {
     return pl->dtype == PACO_C64 && pl->N1 == 256 && pl->N2 == 256 && (pl->p == 4 || pl->p == 8) &&

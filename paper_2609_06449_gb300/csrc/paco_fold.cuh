@@ -11,9 +11,15 @@
 // is multiplied on its way out of a pass, so Phase I stores plain DFTs and the
 // top-level twiddle w_N^{-k1 c} (Sect. 3.3) is taken by Phase III's
 // butterflies.  In complex128, which the FP64 pipe bounds, the count is the
-// time (2^27: 109 operations a point and 27.5 ms with separate products in the
-// stage kernels).  In complex64 it is the issue rate: a pass of 1024 points
-// over 2^28 went from 1.38 ms (139 instructions a point) to 0.76-0.85 ms.
+// time (2^27: 27.5 ms with separate products in the stage kernels, 22.5 ms here).
+// In complex64 it is the issue rate: a pass of 1024 points over 2^28 went from
+// 1.38 ms (139 instructions a point) to 0.79.
+//
+// 2 E - p takes E - t O along where p overflows.  Tiles of such butterflies
+// therefore ask whether their values are that large (may_overflow), and are done
+// again with butterflies whose parts overflow each on its own; or the difference
+// is computed directly, four operations a point and level (Bfly, FoldCfg::BFLY1
+// and BFLY2).
 //
 // A pass transforms L = A B rows (j = j_hi B + j_lo, k = k_lo + A k_hi) of a
 // tile of W columns: A-point DFTs over j_hi in registers, one exchange through
@@ -34,8 +40,7 @@
 // error of 2^24 points is 2.2e-7, with the tables above 1.9e-7 (the stage
 // kernels: 2.0e-7).  2 E - p carries p's rounding on; in FP64, whose error is
 // held to the stage kernels' too, F1 therefore multiplies its rows first and
-// takes the plain DFT (ROWS; 2^27: 21.1 ms, 19.6 with F1 folded at an error 1 to
-// 7 % larger).
+// takes the plain DFT (ROWS), and F2 is direct from three passes on.
 #pragma once
 
 #include "../../include/paco.h"

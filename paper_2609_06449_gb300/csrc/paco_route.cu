@@ -335,9 +335,11 @@ paco_status_t route_setup(paco_plan *pl)
     const int lg[2] = {ilog2_exact(pl->N1), ilog2_exact(pl->N2)}, lgN = lg[0] + lg[1];
     if (pl->form) return pl->dims == 1 ? tc_setup(pl, r, lgN) : PACO_OK;
     int f[MAX_PASSES] = {0, 0, 0, 0};
-    // short transforms: one CTA holds them whole (a few of 2^13 or 2^14 points
-    // spread better over the SMs in two passes: one 2^14 7.9 and 4.9 us, 40 of
-    // them 8.5 and 8.4, 100 8.6 and 10.9)
+    // short transforms: one CTA holds them whole.  2^13 and 2^14 points from a batch
+    // of 32 on: fewer spread better over the SMs in two passes.  us in a graph, whole
+    // and in passes: 2^13 x 1 4.8 and 3.9, x 32 5.3 and 5.0, x 48 5.3 and 5.8, x 128 5.5
+    // and 9.1, x 512 14.6 and 16.1; 2^14 x 1 8.2 and 4.9, x 32 8.7 and 6.0, x 48 8.7
+    // and 9.0, x 128 8.9 and 10.5, x 512 (in L2) 40 and 37.
     const bool whole = pl->dims == 1 && pl->esize == 8 && (lgN < 13 || pl->batch >= 32);
     if (whole && (r->whole = whole_kernel(lgN)).fn) {
         const paco_status_t st = shared_table({pl->device, TABLE_WHOLE, 8, lgN, 0, 0, 0}, &r->tw[0],
