@@ -123,7 +123,7 @@ template <int LG>
 __device__ __forceinline__ void small_item(const BatchedArgs &a, const float2 *tau, int count, const long long *s_off,
                                            unsigned char *smem)
 {
-    whole_tile<WholeCfg<LG, batched::EPT, batched::NT>, batched::EPT, batched::NT>(
+    whole_tile<WholeCfg<LG, batched::EPT, batched::NT, 2 * batched::ITEM>, batched::EPT, batched::NT, false>(
         static_cast<const float2 *>(a.in), static_cast<float2 *>(a.out), a.conj != 0, 1.f, tau,
         [&](int g) { return g < count ? s_off[g] : -1ll; }, reinterpret_cast<cx<float> *>(smem));
 }

@@ -34,6 +34,7 @@ constexpr int DIRECT_LG = 20;      // passes up to K L = 2^20 keep all their fac
 struct Route {
     int n = 0;                     // passes of paco_execute (0: the stage kernels)
     WholeKernel whole;             // n = 1: whole transforms in a CTA
+    WholeKernel whole_scaled;      //   of a scaled input
     FoldKernel k[MAX_PASSES];
     FoldKernel scaled;                 // k[0] for a scaled input (complex64)
     int twmode[MAX_PASSES] = {};       // FoldCfg::TW
@@ -341,11 +342,13 @@ paco_status_t route_setup(paco_plan *pl)
     // and 9.1, x 512 14.6 and 16.1; 2^14 x 1 8.2 and 4.9, x 32 8.7 and 6.0, x 48 8.7
     // and 9.0, x 128 8.9 and 10.5, x 512 (in L2) 40 and 37.
     const bool whole = pl->dims == 1 && pl->esize == 8 && (lgN < 13 || pl->batch >= 32);
-    if (whole && (r->whole = whole_kernel(lgN)).fn) {
+    if (whole && (r->whole = whole_kernel(lgN, false)).fn) {
         const paco_status_t st = shared_table({pl->device, TABLE_WHOLE, 8, lgN, 0, 0, 0}, &r->tw[0],
                                               [&](void **p) { return whole_table(lgN, p); });
         if (st != PACO_OK) return st;
-        PACO_CUDA_TRY(cudaFuncSetAttribute(r->whole.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, r->whole.smem));
+        r->whole_scaled = whole_kernel(lgN, true);
+        for (const WholeKernel *k : {&r->whole, &r->whole_scaled})
+            PACO_CUDA_TRY(cudaFuncSetAttribute(k->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k->smem));
         r->n = 1;
     }
     int n = pl->fused || r->n ? 0 : route_factors(pl, lg[0], lg[1], f);
@@ -437,7 +440,7 @@ paco_status_t route_run(const paco_plan *pl, const void *in, void *out, int dir,
         a.conj = dir == 1;
         a.mult = terms ? terms->ld_mult : 1.f;
         a.scale = terms ? terms->ld_scale : nullptr;
-        return launch(pl, r.whole.fn, &a, (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta, r.whole.threads,
+        return launch(pl, terms ? r.whole_scaled.fn : r.whole.fn, &a, (pl->batch + r.whole.per_cta - 1) / r.whole.per_cta, r.whole.threads,
                       r.whole.smem, false, stream);
     }
     if (pl->form) {

@@ -43,19 +43,22 @@ struct WholeSteps {
     }
 };
 
-template <int LG_, int EPT, int NT>
+// DIRECT_FROM: the length from which the butterflies are DIRECT (whole_step).
+template <int LG_, int EPT, int NT, int DIRECT_FROM = 8192>
 struct WholeCfg {
     using S = WholeSteps<LG_>;
     static constexpr int LG = LG_, N = 1 << LG, TE = EPT * NT, G = TE / N;
     static constexpr int EX0 = G * S::gs(0), EX1 = S::r(2) ? G * S::gs(1) : 0;
     static constexpr int SMEM = (EX0 > EX1 ? EX0 : EX1) * 8;
+    static constexpr bool CARRIES = N > 128 && N < DIRECT_FROM;    // CARRY butterflies
     static_assert(G >= 1 && S::r(0) <= EPT, "tile");
 };
 
 // Step I of the tile's transforms.  off(g): element offset of transform g, or
-// negative where the tile has none; f multiplies the input.  True: nothing was
-// stored, the tile is to be done with AGAIN (may_overflow).
-template <class CFG, int EPT, int NT, int I, bool AGAIN = false, class Off>
+// negative where the tile has none; SCALED: f multiplies the input (as a branch in
+// the one kernel it cost every other call: 2^12 points 0.641 -> 0.650 ms per 2^28).
+// True: nothing was stored, the tile is to be done with AGAIN (may_overflow).
+template <class CFG, int EPT, int NT, int I, bool SCALED, bool AGAIN = false, class Off>
 __device__ __forceinline__ bool whole_step(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
                                            const Off &off, cx<float> *sm)
 {
@@ -63,10 +66,11 @@ __device__ __forceinline__ bool whole_step(const float2 *in, float2 *out, bool c
     using C = cx<float>;
     constexpr int R = S::r(I), K = S::k(I), N = CFG::N, SQ = N / R, U = EPT / R, J = SQ / K;
     constexpr bool LAST = S::r(I + 1) == 0;
-    // Up to 2^7 points the copy rate leaves room for the closer form; above, the
-    // question (may_overflow) costs less: 3001 x 2^12 34.6 -> 35.0 us (DIRECT 35.4),
-    // 200 x 2^13 7.8 -> 8.1 (8.4).
-    constexpr int KIND = AGAIN ? SAFE : N <= 128 ? DIRECT : CARRY;
+    // Up to 2^7 points the copy rate leaves room for the closer form.  Above, the
+    // question (may_overflow) costs less: 2^12 points 0.641 ms per 2^28 without it, 0.642
+    // with it, DIRECT 0.655; but not with 32 points a thread: 2^13 0.698, 0.757, 0.737, 2^14
+    // 0.930, 0.953, 0.945 (the uneven batch keeps the question there, DIRECT spills).
+    constexpr int KIND = AGAIN ? SAFE : !CFG::CARRIES ? DIRECT : CARRY;
     const int tid = threadIdx.x;
     C v[EPT];
     [[maybe_unused]] bool big = false;
@@ -97,7 +101,7 @@ __device__ __forceinline__ bool whole_step(const float2 *in, float2 *out, bool c
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u * R + r] = make_cx<float>(v[u * R + r].y, v[u * R + r].x);
             }
-            if (f != 1.f) {
+            if constexpr (SCALED) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u * R + r] = make_cx<float>(v[u * R + r].x * f, v[u * R + r].y * f);
             }
@@ -133,26 +137,26 @@ __device__ __forceinline__ bool whole_step(const float2 *in, float2 *out, bool c
         } else {
             __syncthreads();
         }
-        whole_step<CFG, EPT, NT, I + 1, AGAIN>(in, out, conj, f, tau, off, sm);
+        whole_step<CFG, EPT, NT, I + 1, SCALED, AGAIN>(in, out, conj, f, tau, off, sm);
     }
     return false;
 }
 
 // The tile with AGAIN, out of line: it takes no register of the common path.
-template <class CFG, int EPT, int NT, class Off>
+template <class CFG, int EPT, int NT, bool SCALED, class Off>
 __device__ __noinline__ void whole_again(const float2 *in, float2 *out, bool conj, float f, const float2 *tau, Off off,
                                          cx<float> *sm)
 {
-    whole_step<CFG, EPT, NT, 0, true>(in, out, conj, f, tau, off, sm);
+    whole_step<CFG, EPT, NT, 0, SCALED, true>(in, out, conj, f, tau, off, sm);
 }
 
 // The tile's transforms, again where they may overflow.
-template <class CFG, int EPT, int NT, class Off>
+template <class CFG, int EPT, int NT, bool SCALED, class Off>
 __device__ __forceinline__ void whole_tile(const float2 *in, float2 *out, bool conj, float f, const float2 *tau,
                                            const Off &off, cx<float> *sm)
 {
-    if (whole_step<CFG, EPT, NT, 0>(in, out, conj, f, tau, off, sm)) {
-        if constexpr (CFG::N > 128) whole_again<CFG, EPT, NT>(in, out, conj, f, tau, off, sm);
+    if (whole_step<CFG, EPT, NT, 0, SCALED>(in, out, conj, f, tau, off, sm)) {
+        if constexpr (CFG::CARRIES) whole_again<CFG, EPT, NT, SCALED>(in, out, conj, f, tau, off, sm);
     }
 }
 
@@ -162,18 +166,18 @@ struct WholeArgs {
     long long batch;
     const float2 *tau;      // the steps' factors (WholeSteps::TAU entries)
     int conj;
-    float mult;             // the input is scaled by mult * (*scale or 1)
+    float mult;             // SCALED: the input is scaled by mult * (*scale or 1)
     const double *scale;
 };
 
-template <int LG, int EPT, int NT>
+template <int LG, int EPT, int NT, bool SCALED>
 __global__ void __launch_bounds__(NT, (EPT == 16 ? 1024 : 512) / NT) paco_whole_kernel(const __grid_constant__ WholeArgs a)
 {
     using CFG = WholeCfg<LG, EPT, NT>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const long long t0 = (long long)blockIdx.x * CFG::G;
-    const float f = a.scale ? a.mult * (float)__ldg(a.scale) : a.mult;
-    whole_tile<CFG, EPT, NT>(
+    const float f = SCALED ? (a.scale ? a.mult * (float)__ldg(a.scale) : a.mult) : 1.f;
+    whole_tile<CFG, EPT, NT, SCALED>(
         a.in, a.out, a.conj != 0, f, a.tau, [&](int g) { return t0 + g < a.batch ? (t0 + g) << LG : -1ll; },
         reinterpret_cast<cx<float> *>(smem_raw));
 }
@@ -183,7 +187,7 @@ struct WholeKernel {
     const void *fn = nullptr;
     int threads = 0, smem = 0, per_cta = 0;
 };
-WholeKernel whole_kernel(int lgN);
+WholeKernel whole_kernel(int lgN, bool scaled);
 
 // The factors of 2^lgN points (device table, paco_route.cu).
 paco_status_t whole_table(int lgN, void **dst);
